@@ -190,6 +190,39 @@ struct Bank {
 #pragma unroll
     for (int i = 0; i < kWords; ++i) w[i * n + s] = t[i];
   }
+  // Stores the words of the fields in MASK (bit i = word i) only.
+  template <unsigned MASK>
+  __device__ __forceinline__ void store_words(int s, const Particle<R>& P) const {
+    Word t[sizeof(Particle<R>) / sizeof(Word)];
+    memcpy(t, &P, sizeof P);
+#pragma unroll
+    for (int i = 0; i < kWords; ++i)
+      if ((MASK >> i) & 1u) w[i * n + s] = t[i];
+  }
+  // the words that hold bytes [off, off + size) of a neutron
+  static __host__ __device__ constexpr unsigned words(size_t off, size_t size) {
+    unsigned m = 0;
+    for (size_t b = off; b < off + size; b += sizeof(int)) m |= 1u << (b / sizeof(Word));
+    return m;
+  }
+  // What an advance with its crossing changes: position, weight, volume, event
+  // counter and last primitive; the direction (a mirror's) and the path length
+  // (timed scorers) in the full build only; the accumulators and the count of
+  // secondaries in gradient runs.
+  template <int OPT>
+  static __host__ __device__ constexpr unsigned moved() {
+    using P = Particle<R>;
+    return words(offsetof(P, x), 3 * sizeof(R)) | words(offsetof(P, w), sizeof(R)) | words(offsetof(P, vol), 4) |
+           words(offsetof(P, k), 4) | words(offsetof(P, last), 4) |
+           ((OPT & kOptFull) ? words(offsetof(P, u), 3 * sizeof(R)) | words(offsetof(P, s), sizeof(R)) : 0u) |
+           (GRAD ? words(offsetof(P, nsec), 4) | words(offsetof(P, A), kMaxPar * sizeof(R)) : 0u);
+  }
+  // What a collision changes: direction, weight, scattering count (and accumulators).
+  static __host__ __device__ constexpr unsigned scattered() {
+    using P = Particle<R>;
+    return words(offsetof(P, u), 3 * sizeof(R)) | words(offsetof(P, w), sizeof(R)) | words(offsetof(P, nscat), 4) |
+           (GRAD ? words(offsetof(P, A), kMaxPar * sizeof(R)) : 0u);
+  }
   // the volume field alone (the regrouping reads it to sort advances)
   __device__ __forceinline__ int vol(int s) const {
     constexpr size_t off = offsetof(Particle<R>, vol);
@@ -589,6 +622,7 @@ template <typename R>
 __device__ __forceinline__ void agg_add2(const AggGroup& G, double* a, double* b, unsigned long long idx, R v,
                                          R v2) {
   int nx = G.next;
+#pragma unroll 1
   for (int k = 0; k < G.rounds; ++k) {
     const int src = nx >= 0 ? nx : (int)(threadIdx.x & 31);
     const R x = __shfl_sync(G.am, v, src);
@@ -682,10 +716,9 @@ __device__ __forceinline__ void score_out(const KParams<R>& kp, const DTally<R>*
       const AggGroup G = agg_group(idx);
       agg_add2(G, kp.sum, kp.sumsq, idx, w, w * w);
       if (GRAD) {
-#pragma unroll
-        for (int p = 0; p < kMaxPar; ++p) {
-          if (p >= kp.npar) break;
-          const R g = w * A[p];
+#pragma unroll 1
+        for (int p = 0; p < kp.npar; ++p) {
+          const R g = w * sel(A, p, R(0));
           agg_add2(G, kp.J, kp.J2, p * stride + idx, g, g * g);
         }
       }
@@ -974,6 +1007,11 @@ struct Adv {
 // WHERE: kAny, or kInPrim / kInWorld when the caller knows where the neutron
 // is (the regrouping kernels), which drops the other branch from the code.
 constexpr int kAny = 0, kInPrim = 1, kInWorld = 2;
+// For cross: either, with a mirror's reflection before the relocation instead of
+// inside it.  The warp pools run the scorer scenes 15 % and the guide 13 % faster
+// this way (5.29e9 against 4.62e9 histories/s total scattering, 1.05e10 against
+// 9.3e9 guide); the history kernel is 25 % slower on total scattering with it.
+constexpr int kPoolCross = 3;
 
 template <typename R, bool GRAD, int OPT, int WHERE = kAny>
 __device__ int advance(const KParams<R>& kp, const View<R>& V, Particle<R>& P, const R (&ip)[kMaxPar], R dR,
@@ -1046,86 +1084,104 @@ __device__ int advance(const KParams<R>& kp, const View<R>& V, Particle<R>& P, c
   return crossing ? kOutCross : kOutColl;
 }
 
-// Relocation at the boundary reached by advance (face / target of `a`).
-// spawn: set when a radius-derivative secondary was created into *S.
-template <typename R, bool GRAD, int OPT, int WHERE = kAny>
-__device__ int cross(const KParams<R>& kp, const View<R>& V, Particle<R>& P, const R (&ip)[kMaxPar], R dR,
-                     unsigned* cnt, int face, int target, Particle<R>* S, bool* spawn) {
-  cnt[C_CROSS]++;
-  if (WHERE == kInPrim || (WHERE == kAny && P.vol >= 0)) {
-    // leave the current primitive: EXIT scorers, then relocate
-    const int from = P.vol;
-    const DPrim<R>& pf = V.prims[from];
-    if (pf.exit_mask) score<R, GRAD, OPT>(kp, V, P, (unsigned)pf.exit_mask, face);
-    const R e = nudge_len(P.x);
-    R xn[3] = {P.x[0] + e * P.u[0], P.x[1] + e * P.u[1], P.x[2] + e * P.u[2]};
-    const int v = locate_after(kp, V, dR, xn, from);
-    P.last = (P.last & kStuckMask) | from | (hull_face(pf.shape, face) ? kLastHull : 0);
-    if (GRAD && !(OPT & kOptNoSec) && kp.radius_par >= 0 && P.sub0 == 0u && pf.shape != TP_BOX &&
-        ((face == 0 && (pf.flags & F_BIND_RMAX)) || (face == 1 && (pf.flags & F_BIND_RMIN)))) {
-      R n[3];
-      normal(pf, P.x, face, n);
-      const int mnext = v >= 0 ? V.prims[v].material : -1;
-      const int mi = face == 0 ? pf.material : mnext;
-      const int mo = face == 0 ? mnext : pf.material;
-      *spawn = radius_crossing<R>(kp, V, P, ip, dR, mi, mo, n, S, cnt);
-    }
-    P.x[0] = xn[0]; P.x[1] = xn[1]; P.x[2] = xn[2];
-    if (v == -2) {
-      if (kp.world_exit_mask) score<R, GRAD, OPT>(kp, V, P, (unsigned)kp.world_exit_mask, -1);
-      return END_ESCAPED;
-    }
-    P.vol = v;
-    if (v >= 0) {
-      const DPrim<R>& pt = V.prims[v];
-      if (pt.entry_mask) score<R, GRAD, OPT>(kp, V, P, (unsigned)pt.entry_mask, -1);
-      if (pt.role == TP_ROLE_DETECTOR) return END_DETECTED;
-      if (pt.role == TP_ROLE_BLACK) return END_BLACK;
-      if ((OPT & kOptFull) && (pt.flags & F_CHOPPER) && !chopper_open(V, pt, P)) return END_BLACK;
-    }
-    return -1;
-  }
-  if (target == -3) {
-    if (kp.world_exit_mask) score<R, GRAD, OPT>(kp, V, P, (unsigned)kp.world_exit_mask, -1);
-    return END_ESCAPED;
-  }
+// Supermirror: weight R(Q), specular reflection (Eq. eMirrowNewDir); the end code or -1.
+template <typename R>
+__device__ __forceinline__ int reflect(const View<R>& V, Particle<R>& P, unsigned* cnt, int face, int target) {
   const DPrim<R>& pt = V.prims[target];
-  if ((OPT & kOptFull) && pt.mirror >= 0) {
-    // supermirror: weight R(Q), specular reflection (Eq. eMirrowNewDir)
-    R n[3];
-    normal(pt, P.x, face, n);
-    const R un = P.u[0] * n[0] + P.u[1] * n[1] + P.u[2] * n[2];
-    const R Q = Tr<R>::kFourPi * fabs(un) / P.lam;
-    const R Rf = mirror_R(V.mirrors[pt.mirror], Q);
-    cnt[C_MIRROR]++;
-    P.w *= Rf;
-    if (!(Rf > R(0))) return END_MIRROR;
+  R n[3];
+  normal(pt, P.x, face, n);
+  const R un = P.u[0] * n[0] + P.u[1] * n[1] + P.u[2] * n[2];
+  const R Q = Tr<R>::kFourPi * fabs(un) / P.lam;
+  const R Rf = mirror_R(V.mirrors[pt.mirror], Q);
+  cnt[C_MIRROR]++;
+  P.w *= Rf;
+  if (!(Rf > R(0))) return END_MIRROR;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) P.u[i] -= R(2) * n[i] * un;
-    P.last = (P.last & kStuckMask) | target | (hull_face(pt.shape, face) ? kLastHull : 0);
-    const R e = nudge_len(P.x);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) P.x[i] += e * P.u[i];
-    return -1;
-  }
-  if (GRAD && !(OPT & kOptNoSec) && kp.radius_par >= 0 && P.sub0 == 0u && pt.shape != TP_BOX &&
-      ((face == 0 && (pt.flags & F_BIND_RMAX)) || (face == 1 && (pt.flags & F_BIND_RMIN)))) {
-    R n[3];
-    normal(pt, P.x, face, n);
-    const int mi = face == 0 ? pt.material : -1;
-    const int mo = face == 0 ? -1 : pt.material;
-    *spawn = radius_crossing<R>(kp, V, P, ip, dR, mi, mo, n, S, cnt);
-  }
+  for (int i = 0; i < 3; ++i) P.u[i] -= R(2) * n[i] * un;
+  P.last = (P.last & kStuckMask) | target | (hull_face(pt.shape, face) ? kLastHull : 0);
   const R e = nudge_len(P.x);
 #pragma unroll
   for (int i = 0; i < 3; ++i) P.x[i] += e * P.u[i];
-  P.vol = target;
-  P.last = (P.last & kStuckMask) | kNoPrim;
-  if (pt.entry_mask) score<R, GRAD, OPT>(kp, V, P, (unsigned)pt.entry_mask, face);
-  if (pt.role == TP_ROLE_DETECTOR) return END_DETECTED;
-  if (pt.role == TP_ROLE_BLACK) return END_BLACK;
-  if ((OPT & kOptFull) && (pt.flags & F_CHOPPER) && !chopper_open(V, pt, P)) return END_BLACK;
   return -1;
+}
+
+// Relocation at the boundary reached by advance (face / target of `a`): out of
+// the current primitive (P.vol >= 0), or from the world region into `target`.
+// spawn: set when a radius-derivative secondary was created into *S.
+//
+// A crossing scores at most twice -- EXIT of the volume it leaves, before it
+// relocates, then ENTRY of the next (or EXIT of the world) -- and both go through
+// one scoring site, the end of a loop over the two parts.  Scoring inlined
+// at each of its five places was half of a kernel's instructions (97 of 212 KB of
+// the lean warp pools), more than the instruction caches hold beside the rest.
+template <typename R, bool GRAD, int OPT, int WHERE = kAny>
+__device__ __forceinline__ int cross(const KParams<R>& kp, const View<R>& V, Particle<R>& P, const R (&ip)[kMaxPar],
+                                     R dR, unsigned* cnt, int face, int target, Particle<R>* S, bool* spawn) {
+  constexpr bool kEither = WHERE == kAny || WHERE == kPoolCross;
+  cnt[C_CROSS]++;
+  const int from = WHERE == kInWorld ? -1 : P.vol;
+  if ((WHERE == kInWorld || WHERE == kPoolCross) && (OPT & kOptFull) && from < 0 && target >= 0 &&
+      V.prims[target].mirror >= 0)
+    return reflect(V, P, cnt, face, target);
+  unsigned mask = WHERE == kInPrim || (kEither && from >= 0) ? (unsigned)V.prims[from].exit_mask : 0u;
+  int sface = face, end = -1;
+#pragma unroll 1
+  for (int part = WHERE == kInWorld ? 1 : 0; part < 2; ++part) {
+    if (part == 1) {
+      mask = 0u;
+      int next = target;   // primitive entered, -1 = world region, < -1 = out of the world
+      if (WHERE == kInPrim || (kEither && from >= 0)) {
+        // leave the current primitive
+        const DPrim<R>& pf = V.prims[from];
+        const R e = nudge_len(P.x);
+        R xn[3] = {P.x[0] + e * P.u[0], P.x[1] + e * P.u[1], P.x[2] + e * P.u[2]};
+        next = locate_after(kp, V, dR, xn, from);
+        P.last = (P.last & kStuckMask) | from | (hull_face(pf.shape, face) ? kLastHull : 0);
+        if (GRAD && !(OPT & kOptNoSec) && kp.radius_par >= 0 && P.sub0 == 0u && pf.shape != TP_BOX &&
+            ((face == 0 && (pf.flags & F_BIND_RMAX)) || (face == 1 && (pf.flags & F_BIND_RMIN)))) {
+          R n[3];
+          normal(pf, P.x, face, n);
+          const int mnext = next >= 0 ? V.prims[next].material : -1;
+          const int mi = face == 0 ? pf.material : mnext;
+          const int mo = face == 0 ? mnext : pf.material;
+          *spawn = radius_crossing<R>(kp, V, P, ip, dR, mi, mo, n, S, cnt);
+        }
+        P.x[0] = xn[0]; P.x[1] = xn[1]; P.x[2] = xn[2];
+        sface = -1;
+      } else if (target >= 0) {
+        const DPrim<R>& pt = V.prims[target];
+        if (WHERE == kAny && (OPT & kOptFull) && pt.mirror >= 0) return reflect(V, P, cnt, face, target);
+        if (GRAD && !(OPT & kOptNoSec) && kp.radius_par >= 0 && P.sub0 == 0u && pt.shape != TP_BOX &&
+            ((face == 0 && (pt.flags & F_BIND_RMAX)) || (face == 1 && (pt.flags & F_BIND_RMIN)))) {
+          R n[3];
+          normal(pt, P.x, face, n);
+          const int mi = face == 0 ? pt.material : -1;
+          const int mo = face == 0 ? -1 : pt.material;
+          *spawn = radius_crossing<R>(kp, V, P, ip, dR, mi, mo, n, S, cnt);
+        }
+        const R e = nudge_len(P.x);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) P.x[i] += e * P.u[i];
+        P.last = (P.last & kStuckMask) | kNoPrim;
+      }
+      if (next < -1) {
+        mask = (unsigned)kp.world_exit_mask;
+        sface = -1;
+        end = END_ESCAPED;
+      } else {
+        P.vol = next;
+        if (next >= 0) {
+          const DPrim<R>& pt = V.prims[next];
+          mask = (unsigned)pt.entry_mask;
+          if (pt.role == TP_ROLE_DETECTOR) end = END_DETECTED;
+          else if (pt.role == TP_ROLE_BLACK) end = END_BLACK;
+          else if ((OPT & kOptFull) && (pt.flags & F_CHOPPER) && !chopper_open(V, pt, P)) end = END_BLACK;
+        }
+      }
+    }
+    if (mask) score<R, GRAD, OPT>(kp, V, P, mask, sface);
+  }
+  return end;
 }
 
 // Interaction at the point reached by advance: process j with probability
@@ -1524,19 +1580,19 @@ __device__ __noinline__ SecCounts run_secondary(const KParams<R>& kp, const View
 }
 
 // The per-slot steps of the regrouping kernels.  A bank (event kernel) or pool
-// (warp-pool kernel) holds one neutron per slot with its next event in pend[];
-// in gradient runs a primary that made a radius-derivative secondary waits in
-// park[] while the secondary runs in its slot.
+// (warp-pool kernel) holds one neutron per slot; its next event is in pend[]
+// (event kernel) or the queue that lists the slot (warp pools).  In gradient
+// runs of the event kernel a primary that made a radius-derivative secondary
+// waits in park[] while the secondary runs in its slot.
 
 // A new history with global index g into `slot`.  Returns -1 if it ended at
 // the source, else 1 if it starts inside a primitive, 0 in the world region.
 template <typename R, bool GRAD, int OPT>
-__device__ __forceinline__ int slot_start(const KParams<R>& kp, const View<R>& V, const Bank<R, GRAD>& bank, int* pend,
-                                          int slot, unsigned long long g, unsigned* cnt) {
+__device__ __forceinline__ int new_history(const KParams<R>& kp, const View<R>& V, const Bank<R, GRAD>& bank, int slot,
+                                           unsigned long long g, unsigned* cnt) {
   if (kp.sec_mode == 2) {   // a queued secondary: it starts where it was made
     const Particle<R> S = sec_read(reinterpret_cast<const SecRec<R>*>(kp.sec_buf) + g);
     bank.store(slot, S);
-    pend[slot] = EV_ADV;
     return S.vol >= 0 ? 1 : 0;
   }
   g += kp.index_base;
@@ -1558,17 +1614,24 @@ __device__ __forceinline__ int slot_start(const KParams<R>& kp, const View<R>& V
     return -1;
   }
   bank.store(slot, P);
-  pend[slot] = EV_ADV;
   return P.vol >= 0 ? 1 : 0;
+}
+
+// The same with the slot's next event noted (event kernel).
+template <typename R, bool GRAD, int OPT>
+__device__ __forceinline__ int slot_start(const KParams<R>& kp, const View<R>& V, const Bank<R, GRAD>& bank, int* pend,
+                                          int slot, unsigned long long g, unsigned* cnt) {
+  const int born = new_history<R, GRAD, OPT>(kp, V, bank, slot, g, cnt);
+  if (born >= 0) pend[slot] = EV_ADV;
+  return born;
 }
 
 // Advance the neutron of `slot` and, if it reaches a boundary, cross it (inside
 // a primitive every crossing is an exit, in the world region an entry; the
 // caller knows which: in_prim).  Returns true if it now waits for a collision.
-// PARK: a secondary that is not queued takes over the slot while its primary
-// waits in park[] (event kernel); without PARK (warp pools) the lane runs it
-// to its end at once, out of line, and the pool needs no parking bank.
-template <typename R, bool GRAD, int OPT, bool PARK = true>
+// A secondary that is not queued takes over the slot while its primary waits
+// in park[].
+template <typename R, bool GRAD, int OPT>
 __device__ __forceinline__ bool slot_advance(const KParams<R>& kp, const View<R>& V, const Bank<R, GRAD>& bank,
                                              const Bank<R, GRAD>& park, int* pend, int* parked, int slot, bool in_prim,
                                              unsigned* cnt) {
@@ -1592,18 +1655,12 @@ __device__ __forceinline__ bool slot_advance(const KParams<R>& kp, const View<R>
   } else {
     if (end >= 0) finish(kp, P, end);
     if (GRAD && spawn && sec_push(kp, S)) spawn = false;
-    if (GRAD && !PARK && spawn) {
-      const SecCounts r = run_secondary<R, OPT>(kp, V, S, ip, dR);
-#pragma unroll
-      for (int i = 0; i < kNumCounters; ++i) cnt[i] += r.c[i];
-      spawn = false;
-    }
-    if (GRAD && PARK && spawn) {
+    if (GRAD && spawn) {
       if (end < 0) { park.store(slot, P); parked[slot] = 1; }
       P = S;
       pend[slot] = EV_ADV;
     } else if (end >= 0) {
-      if (GRAD && PARK && parked[slot]) { P = park.load(slot); parked[slot] = 0; pend[slot] = EV_ADV; }
+      if (GRAD && parked[slot]) { P = park.load(slot); parked[slot] = 0; pend[slot] = EV_ADV; }
       else pend[slot] = EV_EMPTY;
     } else {
       pend[slot] = EV_ADV;
@@ -1614,7 +1671,7 @@ __device__ __forceinline__ bool slot_advance(const KParams<R>& kp, const View<R>
 }
 
 // The collision the neutron of `slot` waits for.
-template <typename R, bool GRAD, bool PARK = true>
+template <typename R, bool GRAD>
 __device__ __forceinline__ void slot_collide(const KParams<R>& kp, const View<R>& V, const Bank<R, GRAD>& bank,
                                              const Bank<R, GRAD>& park, int* pend, int* parked, int slot,
                                              unsigned* cnt) {
@@ -1624,7 +1681,7 @@ __device__ __forceinline__ void slot_collide(const KParams<R>& kp, const View<R>
   const int end = collide_again<R, GRAD>(kp, V, P, ip, cnt);
   if (end >= 0) {
     finish(kp, P, end);
-    if (GRAD && PARK && parked[slot]) { P = park.load(slot); parked[slot] = 0; pend[slot] = EV_ADV; }
+    if (GRAD && parked[slot]) { P = park.load(slot); parked[slot] = 0; pend[slot] = EV_ADV; }
     else pend[slot] = EV_EMPTY;
   } else {
     pend[slot] = EV_ADV;
@@ -1827,13 +1884,78 @@ __global__ void __launch_bounds__(256, MINB) k_transport_ev(const __grid_constan
 // entry crossing --, collision) on up to 32 of them, so the warp executes one
 // code path with most lanes busy.  Warps never wait for one another: no CTA
 // barrier after the table copy.
+//
+// What bounds it is the supply of instructions: a step runs some 650 of them
+// once each, the warps of an SM are at different places of the code, and the
+// fetch stall is the first of all (3.8 of 11 cycles an instruction on the powder
+// scene, 4.9 of 13 before).  Hence few of them: a step's slots come off a
+// stack, not out of a search of the pool, and a step writes back only the words
+// it changes.
+//
+// Queues: each event type has a stack of slot numbers; the counts are one
+// packed word (a byte each) that every lane holds.  A step pops up to 32 slots
+// from the fullest stack and pushes each to the stack of its next event.  Last
+// in, first out keeps the neutrons of a step together -- started together,
+// they are mostly in the same volume and test the same surfaces.  Powder /
+// total scattering / guide / biased FP32 slab / imaging at 1e8, 4e7, 1e8, 4e7
+// and 1e7 histories, in 1e9 histories/s: 5.10 / 4.38 / 9.04 / 3.77 / 0.93 with
+// slots picked from the pool's event words by ballots and scoring at five
+// places, 5.78 / 5.29 / 10.5 / 4.12 / 1.05 with the stacks and one scoring
+// site; with the queues first in, first out 4.79 / 3.88 / 9.40 / 3.79 / 1.02;
+// with two warps of a sub-partition on a pool in common, so that one fetch may
+// serve both, 4.88 / 4.85 / 8.48 / 4.48 / 1.03.
 // ---------------------------------------------------------------------------
-#ifndef TP_POOL
-#define TP_POOL 64
-#endif
-constexpr int kPool = TP_POOL;            // neutrons per warp (a multiple of 32)
-static_assert(kPool % 32 == 0, "pool size");
-constexpr int kPoolGroups = kPool / 32;   // pool slots per lane
+constexpr int kPool = 64;   // neutrons per warp (the stacks' counts are bytes)
+
+// byte q of a packed word
+__device__ __forceinline__ int byte_of(unsigned v, int q) { return (int)__byte_perm(v, 0u, 0x4440u | (unsigned)q); }
+
+// Advance the neutron of `slot` and cross the boundary it reaches, if any;
+// returns the queue of its next event.  A radius-derivative secondary that is
+// not queued for the second pass is run to its end at once, out of line, so that
+// the pool needs no parking place.
+template <typename R, bool GRAD, int OPT>
+__device__ __forceinline__ int pool_advance(const KParams<R>& kp, const View<R>& V, const Bank<R, GRAD>& pool, int slot,
+                                            bool in_prim, unsigned* cnt) {
+  Particle<R> P = pool.load(slot);
+  R ip[kMaxPar], dR;
+  load_params(kp, P.inst, ip, &dR);
+  Adv<R> a;
+  bool spawn = false;
+  Particle<R> S;
+  int end;
+  if (in_prim) end = advance<R, GRAD, OPT, kInPrim>(kp, V, P, ip, dR, cnt, a);
+  else end = advance<R, GRAD, OPT, kInWorld>(kp, V, P, ip, dR, cnt, a);
+  if (end == kOutCross) end = cross<R, GRAD, OPT, kPoolCross>(kp, V, P, ip, dR, cnt, a.face, a.target, &S, &spawn);
+  int next = Q_COLL;
+  if (end != kOutColl) {
+    if (end >= 0) finish(kp, P, end);
+    if (GRAD && spawn && !sec_push(kp, S)) {
+      const SecCounts r = run_secondary<R, OPT>(kp, V, S, ip, dR);
+#pragma unroll
+      for (int i = 0; i < kNumCounters; ++i) cnt[i] += r.c[i];
+    }
+    next = end >= 0 ? Q_EMPTY : (P.vol >= 0 ? Q_ADVP : Q_ADVW);
+  }
+  pool.template store_words<Bank<R, GRAD>::template moved<OPT>()>(slot, P);
+  return next;
+}
+
+// The collision the neutron of `slot` waits for; returns the queue of its next event.
+template <typename R, bool GRAD>
+__device__ __forceinline__ int pool_collide(const KParams<R>& kp, const View<R>& V, const Bank<R, GRAD>& pool, int slot,
+                                            unsigned* cnt) {
+  Particle<R> P = pool.load(slot);
+  R ip[kMaxPar], dR;
+  load_params(kp, P.inst, ip, &dR);
+  const int end = collide_again<R, GRAD>(kp, V, P, ip, cnt);
+  if (end >= 0) {
+    finish(kp, P, end);
+    return Q_EMPTY;
+  }
+  pool.template store_words<Bank<R, GRAD>::scattered()>(slot, P);
+  return Q_ADVP;
+}
 
 template <typename R, bool GRAD, int OPT, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_transport_wq(const __grid_constant__ KParams<R> kp) {
@@ -1862,117 +1984,71 @@ __global__ void __launch_bounds__(256, MINB) k_transport_wq(const __grid_constan
   const int lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
   const int warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
-  __shared__ unsigned char sel[8][32];   // per warp: the slots of this step, in lane order
-  unsigned char* sel_row = sel[warp];
-  // per warp: its pool of kPool neutrons and their pending event types (no
-  // parking: a secondary that is not queued runs to its end at once)
+  // per warp: its pool of kPool neutrons (no parking: a secondary that is not
+  // queued runs to its end at once) and a stack of kPool slots per queue
   using BankT = Bank<R, GRAD>;
   const BankT pool(smem + tab + BankT::bytes(kPool) * warp, kPool);
-  const BankT park = pool;   // unused (PARK false)
-  int* pend = reinterpret_cast<int*>(smem + tab + BankT::bytes(kPool) * nwarps) + warp * 2 * kPool;
-  int* parked = pend + kPool;
+  uint8_t* stack = smem + tab + BankT::bytes(kPool) * (blockDim.x >> 5) + kNumQ * kPool * warp;
 
   const unsigned long long total = work_total(kp);
   unsigned cnt[kNumCounters];   // per-thread counts: 32 bits suffice (widened below)
 #pragma unroll
   for (int i = 0; i < kNumCounters; ++i) cnt[i] = 0;
   unsigned polls = 0;   // claims made by this thread (abort polling)
+  // every slot is free
 #pragma unroll
-  for (int g = 0; g < kPoolGroups; ++g) { pend[g * 32 + lane] = EV_EMPTY; parked[g * 32 + lane] = 0; }
-  __syncwarp();
-  unsigned long long chunk_next = 0, chunk_end = 0;   // warp-uniform
-  bool work_left = true;                              // warp-uniform
+  for (int i = 0; i < kPool; i += 32) stack[Q_EMPTY * kPool + i + lane] = (uint8_t)(i + lane);
+  unsigned counts = (unsigned)kPool << (8 * Q_EMPTY);   // warp-uniform
+  bool work_left = true;                                // warp-uniform
 
   for (;;) {
-    // ---- count what the pool waits for ----
-    unsigned m[kNumQ][kPoolGroups];
-#pragma unroll
-    for (int g = 0; g < kPoolGroups; ++g) {
-      const int slot = g * 32 + lane;
-      const int ty = pend[slot];
-      const bool adv = ty == EV_ADV;
-      const bool inprim = adv && pool.vol(slot) >= 0;
-      m[Q_EMPTY][g] = __ballot_sync(kFull, ty == EV_EMPTY);
-      m[Q_ADVP][g] = __ballot_sync(kFull, adv && inprim);
-      m[Q_ADVW][g] = __ballot_sync(kFull, adv && !inprim);
-      m[Q_COLL][g] = __ballot_sync(kFull, ty == EV_COLL);
-    }
-    int count[kNumQ];
-#pragma unroll
-    for (int q = 0; q < kNumQ; ++q) {
-      count[q] = 0;
-#pragma unroll
-      for (int g = 0; g < kPoolGroups; ++g) count[q] += __popc(m[q][g]);
-    }
+    __syncwarp();   // the last step's pushes and stores
     // ---- pick the queue: refill when half the pool is free, else the fullest ----
-    int q = -1;
-    if (work_left && count[Q_EMPTY] >= 32) {
+    int q = -1, best = 0;
+    if (work_left && byte_of(counts, Q_EMPTY) >= 32) {
       q = Q_EMPTY;
     } else {
-      int best = 0;
 #pragma unroll
       for (int k = 1; k < kNumQ; ++k)
-        if (count[k] > best) { best = count[k]; q = k; }
+        if (byte_of(counts, k) > best) { best = byte_of(counts, k); q = k; }
       if (q < 0) {
-        if (work_left && count[Q_EMPTY] > 0) q = Q_EMPTY;
-        else break;   // nothing live and no work left
+        if (!work_left || byte_of(counts, Q_EMPTY) == 0) break;   // nothing live and no work left
+        q = Q_EMPTY;
       }
     }
-    // ---- lane j takes the j-th slot of queue q ----
-    const int n = min(count[q], 32);
+    // ---- lane j takes the j-th of the top entries ----
+    const int n = min(byte_of(counts, q), 32);
+    counts -= (unsigned)n << (8 * q);
     int slot = -1;
-    if constexpr (!(OPT & kOptFull)) {
-      // lean build: the slots' own lanes write their indices in rank order to
-      // the warp's selection row and lane j reads entry j (powder +14 %)
-      int base = 0;
-#pragma unroll
-      for (int g = 0; g < kPoolGroups; ++g) {
-        const unsigned mg = m[q][g];
-        const int r = base + __popc(mg & lt_mask);
-        if (((mg >> lane) & 1u) && r < 32) sel_row[r] = (unsigned char)(g * 32 + lane);
-        base += __popc(mg);
-      }
-      __syncwarp();
-      if (lane < n) slot = (int)sel_row[lane];
-      __syncwarp();
-    } else if (lane < n) {
-      // full build: each lane finds its set bit (guide and total scattering
-      // run 5 % faster this way)
-      int j = lane;
-#pragma unroll
-      for (int g = 0; g < kPoolGroups; ++g) {
-        const int c = __popc(m[q][g]);
-        if (slot < 0) {
-          if (j < c) slot = g * 32 + (int)__fns(m[q][g], 0, j + 1);
-          else j -= c;
-        }
-      }
-    }
+    if (lane < n) slot = stack[q * kPool + byte_of(counts, q) + lane];
+    int to = -1;   // queue of the slot's next event
     if (q == Q_EMPTY) {
-      // new histories from the warp's chunk of global indices
-      int taken = 0;
-      while (taken < n) {
-        if (chunk_next >= chunk_end) {
-          unsigned long long b = 0;
-          if (lane == 0) b = aborted(kp, polls) ? total : atomicAdd(kp.work_counter, (unsigned long long)kp.chunk);
-          b = __shfl_sync(kFull, b, 0);
-          if (b >= total) { work_left = false; break; }
-          chunk_next = b;
-          chunk_end = min(b + (unsigned long long)kp.chunk, total);
+      // new histories, claimed for the whole step at once
+      unsigned long long g = 0;
+      if (lane == 0) g = aborted(kp, polls) ? total : atomicAdd(kp.work_counter, (unsigned long long)n);
+      g = __shfl_sync(kFull, g, 0) + lane;
+      if (slot >= 0) {
+        to = Q_EMPTY;
+        if (g < total) {
+          const int born = new_history<R, GRAD, OPT>(kp, V, pool, slot, g, cnt);
+          if (born >= 0) to = born == 1 ? Q_ADVP : Q_ADVW;
         }
-        const int avail = (int)min((unsigned long long)(n - taken), chunk_end - chunk_next);
-        if (lane >= taken && lane < taken + avail)
-          slot_start<R, GRAD, OPT>(kp, V, pool, pend, slot, chunk_next + (lane - taken), cnt);
-        chunk_next += avail;
-        taken += avail;
       }
-    } else if (q == Q_ADVP || q == Q_ADVW) {
-      if (slot >= 0) slot_advance<R, GRAD, OPT, false>(kp, V, pool, park, pend, parked, slot, q == Q_ADVP, cnt);
-    } else {
-      if (slot >= 0) slot_collide<R, GRAD, false>(kp, V, pool, park, pend, parked, slot, cnt);
+      work_left = __all_sync(kFull, slot < 0 || g < total) != 0;
+    } else if (slot >= 0) {
+      if (q == Q_COLL) to = pool_collide<R, GRAD>(kp, V, pool, slot, cnt);
+      else to = pool_advance<R, GRAD, OPT>(kp, V, pool, slot, q == Q_ADVP, cnt);
     }
-    __syncwarp();
+    // ---- push each slot to the stack of its next event ----
+    unsigned added = 0u, mine = 0u;
+#pragma unroll
+    for (int k = 0; k < kNumQ; ++k) {
+      const unsigned m = __ballot_sync(kFull, to == k);
+      added |= (unsigned)__popc(m) << (8 * k);
+      if (to == k) mine = m;
+    }
+    if (to >= 0) stack[to * kPool + byte_of(counts, to) + __popc(mine & lt_mask)] = (uint8_t)slot;
+    counts += added;
   }
 #pragma unroll
   for (int i = 0; i < kNumCounters; ++i) {
@@ -2203,7 +2279,7 @@ size_t bank_bytes(int variant, int precision, bool grad, int block) {
     return ps * block * (grad ? 2 : 1) + 2 * sizeof(int) * block + sizeof(unsigned short) * kNumQMax * block;
   if (variant == TP_KERNEL_WARPQ) {
     const size_t slots = (size_t)(block / 32) * kPool;
-    return ps * slots + 2 * sizeof(int) * slots;
+    return ps * slots + kNumQ * slots;   // the pools and their stacks
   }
   return 0;
 }
