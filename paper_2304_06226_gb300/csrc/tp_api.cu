@@ -103,7 +103,10 @@ struct LaunchCfg {
   int defer;   // gradient runs: secondaries queued and transported in a second pass
   int full = 1;  // the build with every feature (else the lean one)
   int regroup = 1;  // event kernel, plain runs: events between regroupings
-  int variant() const { return kernel | (hi ? kVariantHighOcc : 0) | (full ? kVariantFull : 0); }
+  int count = 0;    // warp pools, plain runs: tallies counted in shared memory
+  int variant() const {
+    return kernel | (hi ? kVariantHighOcc : 0) | (full ? kVariantFull : 0) | (count ? kVariantCount : 0);
+  }
 };
 
 struct tp_scene {
@@ -117,6 +120,7 @@ struct tp_scene {
   int full = 1;
   int full_needed = 1;   // what the description needs (full may be forced by a test flag)
   int src_free = 0;      // every source point in the world region (set with the tables)
+  int world_clear = 0;   // every primitive well inside the world (set with the tables)
   // description (owned copies)
   int world_shape = TP_BOX;
   double world_c[3] = {0, 0, 0}, world_p[3] = {0, 0, 0};
@@ -454,9 +458,35 @@ bool source_in_free_space(const tp_scene* s) {
   return true;
 }
 
+// True if every primitive (every instance) keeps a margin far above the
+// transport precision's rounding and nudges from the world's boundary: whatever
+// a ray meets then comes before the boundary.
+bool prims_clear_of_world(const tp_scene* s) {
+  double scale = 1.0;
+  for (int k = 0; k < 3; ++k)
+    scale = std::max(scale, std::fabs(s->world_c[k]) + (s->world_shape == TP_BOX ? s->world_p[k] : s->world_p[1]));
+  const double m = 1e-3 * scale;
+  bool moving = false;
+  for (const auto& p : s->prims) moving |= (p.bind_rmin || p.bind_rmax);
+  const int ninst = moving ? s->n_inst : 1;
+  for (const auto& p : s->prims)
+    for (int q = 0; q < ninst; ++q) {
+      const Box3 b = aabb(s, p, q);
+      double far2 = 0;
+      for (int k = 0; k < 3; ++k) {
+        const double e = std::max(std::fabs(b.lo[k] - s->world_c[k]), std::fabs(b.hi[k] - s->world_c[k]));
+        if (s->world_shape == TP_BOX && e + m >= s->world_p[k]) return false;
+        far2 += e * e;
+      }
+      if (s->world_shape != TP_BOX && std::sqrt(far2) + m >= s->world_p[1]) return false;
+    }
+  return true;
+}
+
 template <typename R>
 std::vector<uint8_t> build_blob(tp_scene* s) {
   s->src_free = source_in_free_space(s) ? 1 : 0;
+  s->world_clear = prims_clear_of_world(s) ? 1 : 0;
   const int np = (int)s->prims.size(), nm = (int)s->mats.size(), nmir = (int)s->mirrors.size(),
             nch = (int)s->choppers.size(), nt = (int)s->tallies.size();
   int nl = 0;
@@ -708,6 +738,7 @@ void fill_common(const tp_scene* s, KParams<R>& k) {
       if (s->tallies[t].trigger == TP_PTS_EXIT) k.world_exit_mask |= 1 << t;
       else k.world_entry_mask |= 1 << t;
     }
+  k.world_free = s->world_clear && k.world_exit_mask == 0 ? 1 : 0;
   const tp_source& src = s->source;
   k.src_kind = src.kind;
   k.src_aperture = src.has_aperture;
@@ -763,8 +794,26 @@ tp_status pick_launch(tp_scene* s, bool grad, int req_block, int req_ctas, int* 
   return TP_OK;
 }
 
+// Bins of a histogram in shared memory: 16 KB a block leave the warp pools
+// their four blocks of 256 threads per SM (54 of 57 KB a block).
+constexpr int kCountBinsMax = 4096;
+
+// True if plain runs of the warp pools may count instead of summing weights: no
+// process is biased and no surface reflects, so every weight stays exactly 1.
+bool counts_only(const tp_scene* s) {
+  if (s->n_inst != 1 || s->total_bins < 1 || s->total_bins > kCountBinsMax || s->grid_cells > 0) return false;
+  for (const tp_prim& p : s->prims)
+    if (p.mirror >= 0) return false;
+  for (const Mat& m : s->mats)
+    for (double g : m.g)
+      if (g != 1.0) return false;
+  return true;
+}
+
+// variant: the kernel, with kVariantCount if it counts.
 size_t smem_variant(const tp_scene* s, int variant, bool grad, int block, int stage) {
-  return (stage ? align16(s->blob_bytes) : 0) + align16(bank_bytes(variant, s->precision, grad, block));
+  return (stage ? align16(s->blob_bytes) : 0) + align16(bank_bytes(variant, s->precision, grad, block)) +
+         ((variant & kVariantCount) ? align16(sizeof(unsigned) * (size_t)s->total_bins) : 0);
 }
 
 // Tables larger than this are offered to the autotuner unstaged as well
@@ -775,8 +824,10 @@ constexpr uint32_t kStageChoiceBytes = 16 * 1024;
 // stage: -1 = stage the tables when they fit (<= kMaxStagedBlob).
 // hi: -1 = the 80-register build unless req_ctas asks for more CTAs per SM
 // than it allows and the 64-register build allows more; 0 / 1 = that build.
+// weighted: a launch whose weights are not those of the scene's own histories
+// (the second pass over queued secondaries), which never counts.
 tp_status resolve(tp_scene* s, bool grad, int kernel, int req_block, int req_ctas, LaunchCfg* c, int stage = -1,
-                  int hi = -1) {
+                  int hi = -1, bool weighted = false) {
   const int b = req_block > 0 ? req_block : 256;
   if (b % 32 != 0 || b < 32 || b > 256)
     return fail(TP_ERR_INVALID_ARG, "kernel %d block_size %d: need a multiple of 32 in [32, 256]", kernel, b);
@@ -786,17 +837,19 @@ tp_status resolve(tp_scene* s, bool grad, int kernel, int req_block, int req_cta
     TP_CUDA(cudaDeviceGetAttribute(&s->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   }
   const size_t limit = (size_t)s->smem_optin;
+  const int count = kernel == TP_KERNEL_WARPQ && !grad && !weighted && counts_only(s) ? 1 : 0;
+  const int form = kernel | (count ? kVariantCount : 0);
   // stage the tables when they are small enough and fit beside the neutron bank
-  if (stage < 0) stage = s->blob_bytes <= kMaxStagedBlob && smem_variant(s, kernel, grad, b, 1) <= limit ? 1 : 0;
+  if (stage < 0) stage = s->blob_bytes <= kMaxStagedBlob && smem_variant(s, form, grad, b, 1) <= limit ? 1 : 0;
   if (stage && s->blob_bytes > kMaxStagedBlob) return fail(TP_ERR_INVALID_ARG, "tables too large to stage");
-  if (smem_variant(s, kernel, grad, b, stage) > limit)
+  if (smem_variant(s, form, grad, b, stage) > limit)
     return fail(TP_ERR_INVALID_ARG, "kernel %d block_size %d needs %zu bytes of shared memory; a block may use %zu",
-                kernel, b, smem_variant(s, kernel, grad, b, stage), limit);
+                kernel, b, smem_variant(s, form, grad, b, stage), limit);
   const bool can_hi = s->precision == TP_FP32;
   if (hi > 0 && !can_hi) return fail(TP_ERR_INVALID_ARG, "the 64-register build serves FP32 runs only");
   int h = hi > 0 ? 1 : 0, occ = 0;
-  const size_t sm = smem_variant(s, kernel, grad, b, stage);
-  const int fbit = s->full ? kVariantFull : 0;
+  const size_t sm = smem_variant(s, form, grad, b, stage);
+  const int fbit = (s->full ? kVariantFull : 0) | (count ? kVariantCount : 0);
   TP_CUDA(occupancy_transport(kernel | (h ? kVariantHighOcc : 0) | fbit, s->precision, grad, s->grid_cells > 0, b, sm, &occ));
   if (hi < 0 && can_hi && req_ctas > occ) {
     int occ_hi = 0;
@@ -804,7 +857,7 @@ tp_status resolve(tp_scene* s, bool grad, int kernel, int req_block, int req_cta
     if (occ_hi > occ) { h = 1; occ = occ_hi; }
   }
   if (occ < 1) return fail(TP_ERR_INVALID_ARG, "kernel %d block_size %d does not fit on an SM", kernel, b);
-  *c = LaunchCfg{kernel, b, req_ctas > 0 ? std::min(req_ctas, occ) : occ, stage, h, 0, s->full};
+  *c = LaunchCfg{kernel, b, req_ctas > 0 ? std::min(req_ctas, occ) : occ, stage, h, 0, s->full, 1, count};
   return TP_OK;
 }
 
@@ -839,7 +892,7 @@ cudaError_t launch_one(tp_scene* s, const LaunchCfg& c, bool grad, uint64_t seed
   k.chunk = sec_mode == 2 ? 16 : (int)std::max(1ll, std::min(256ll, (long long)(total / (unsigned long long)(warps * 8))));
   cudaError_t e = cudaMemsetAsync(s->d_work, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  const size_t sm = smem_variant(s, c.kernel, grad, c.block, c.stage);
+  const size_t sm = smem_variant(s, c.variant(), grad, c.block, c.stage);
   if constexpr (std::is_same<R, double>::value) return launch_transport_f64(k, c.variant(), grad, grid, c.block, sm, st);
   else return launch_transport_f32(k, c.variant(), grad, grid, c.block, sm, st);
 }
@@ -863,7 +916,7 @@ tp_status ensure_sec(tp_scene* s, unsigned long long total) {
   unsigned long long want = kSecCapMin;
   while (want < cap && want < kSecPerHistory * total && 2 * want <= mem_cap) want <<= 1;
   if (s->sec_cfg.kernel == 0) {
-    tp_status st = resolve(s, false, TP_KERNEL_WARPQ, 256, 0, &s->sec_cfg, -1, s->precision == TP_FP32 ? 1 : 0);
+    tp_status st = resolve(s, false, TP_KERNEL_WARPQ, 256, 0, &s->sec_cfg, -1, s->precision == TP_FP32 ? 1 : 0, true);
     if (st != TP_OK) return st;
   }
   if (s->d_sec && s->sec_cap >= want && s->sec_cap <= cap) return TP_OK;

@@ -90,6 +90,7 @@ struct KParams {
   int world_shape;
   R world_c[3], world_p[3];
   int world_entry_mask, world_exit_mask;
+  int world_free;   // 1: no tally listens to the world's EXIT and every primitive keeps clear of its boundary
   // source
   int src_kind, src_aperture;
   R src_c[3], src_half[2], src_lam_lo, src_lam_hi, src_div[2], src_ap[2];
@@ -150,6 +151,10 @@ struct KParams {
 // lean build, for scenes that use none of them).
 constexpr int kVariantHighOcc = 16;
 constexpr int kVariantFull = 32;
+// kVariantCount (warp pools, plain runs, one instance, no grid): the weights of
+// the scene stay 1 and its bins fit beside the pools, so the tallies are counted
+// in shared memory.
+constexpr int kVariantCount = 64;
 cudaError_t launch_transport_f32(const KParams<float>& p, int variant, bool grad, int grid, int block,
                                  size_t smem, cudaStream_t st);
 cudaError_t launch_transport_f64(const KParams<double>& p, int variant, bool grad, int grid, int block,

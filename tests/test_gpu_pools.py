@@ -1,0 +1,82 @@
+"""The warp pools at the edges of their steps: fewer histories than lanes, one
+step's worth, a pool's worth and one more, blocks of one warp to eight.  FP64,
+against the history kernel: every history has its own random numbers, so the
+counters agree exactly and the tallies to the rounding of their sums (at most
+a few thousand FP64 additions of like sign: 1e-12)."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(desc, n, kernel, block, grad=False):
+    from paper_2304_06226_gb300.engine import Scene
+    sc = Scene(desc)
+    sc.run(n, kernel=kernel, block_size=block, want_grad=grad, secondaries=2 if grad else 0)
+    torch.cuda.synchronize()
+    raw = [sc.raw(q) for q in range(sc.n_inst)]
+    cnt = sc.counters()
+    sc.close()
+    return cnt, {k: np.stack([r[k] for r in raw]) for k in ("sum", "sumsq", "J")}
+
+
+SCENES = {"powder": lambda: W.powder(precision="f64", g=(0.5, 2.0, 2.0)), "guide": lambda: W.guide(precision="f64"),
+          "slab": lambda: W.slab(g=3.0), "chopper": lambda: W.chopper(precision="f64"),
+          "batched": lambda: W.batched(n_instances=3, precision="f64"),
+          "imaging": lambda: W.imaging(n_prims=60, precision="f64", psd_bins=16)}
+
+
+@pytest.mark.parametrize("block", [32, 160, 256])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 64, 65, 4097])
+@pytest.mark.parametrize("scene", sorted(SCENES))
+def test_pool_steps(scene, n, block):
+    desc = SCENES[scene]()
+    grad = scene in ("batched", "imaging")
+    cnt, got = _run(desc, n, 3, block, grad)
+    ref_cnt, ref = _run(desc, n, 1, 128, grad)
+    assert cnt == ref_cnt
+    for k, v in ref.items():
+        if v.size:
+            assert np.allclose(got[k], v, rtol=1e-12, atol=1e-12 * max(1e-300, np.abs(v).max())), k
+
+
+# Scenes whose weights stay 1: the pools count in shared memory, the event
+# kernel adds w and w^2 with FP64 atomics; both are whole numbers and equal.
+# 4096 bins are the most a histogram holds; with one more the pools add weights.
+UNIT = {"powder": lambda p: W.powder(precision=p), "powder_4096": lambda p: W.powder(precision=p, nbins=4096),
+        "powder_4097": lambda p: W.powder(precision=p, nbins=4097),
+        "orders": lambda p: W.total_scattering(precision=p, g=1.0),
+        "chopper": lambda p: W.chopper(precision=p), "slit": lambda p: W.moderator_test(precision=p, temperature=300.0),
+        "slab": lambda p: W.slab(g=1.0, precision=p)}
+
+
+@pytest.mark.parametrize("n", [1, 100, 50_001])
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+@pytest.mark.parametrize("scene", sorted(UNIT))
+def test_counting_equals_summing(scene, precision, n):
+    desc = UNIT[scene](precision)
+    cnt, got = _run(desc, n, 3, 256)
+    ref_cnt, ref = _run(desc, n, 2, 256)
+    assert cnt == ref_cnt
+    assert (got["sum"] == ref["sum"]).all() and (got["sumsq"] == ref["sumsq"]).all()
+    assert (got["sum"] == np.rint(got["sum"])).all() and (got["sum"] == got["sumsq"]).all()
+
+
+def test_counting_adds_to_what_is_there_and_stops_with_a_bias():
+    from paper_2304_06226_gb300.engine import Scene
+    sc = Scene(W.powder())
+    sc.run(1000, kernel=3, first=0)
+    sc.run(1000, kernel=3, first=1000)
+    two = sc.raw()["sum"].copy()
+    sc.reset()
+    sc.run(2000, kernel=3)
+    assert (sc.raw()["sum"] == two).all()
+    sc.reset()
+    sc.set_bias(0, (1.0, 2.0, 1.0))   # weights now differ from 1
+    sc.run(20_000, kernel=3)
+    raw = sc.raw()
+    sc.close()
+    assert not (raw["sum"] == raw["sumsq"]).all()
