@@ -146,6 +146,8 @@ struct tp_scene {
   bool blob_dirty = true;
   // uniform grid (scenes with more than kGridMinPrims primitives)
   int* d_grid = nullptr;   // [ncells + 1] starts, then items
+  void* d_grid_rows = nullptr;   // the items' bounding spheres (GridRow)
+  std::vector<int> grid_items;   // host copy of the items
   int grid_n[3] = {0, 0, 0};
   double grid_lo[3] = {0, 0, 0}, grid_hi[3] = {0, 0, 0};
   int grid_cells = 0;
@@ -593,7 +595,9 @@ constexpr double kGridCellsPerPrim = 1.0;
 // (over every instance) meets it.
 tp_status upload_grid(tp_scene* s) {
   if (s->d_grid) { cudaFree(s->d_grid); s->d_grid = nullptr; }
+  if (s->d_grid_rows) { cudaFree(s->d_grid_rows); s->d_grid_rows = nullptr; }
   s->grid_cells = 0;
+  s->grid_items.clear();
   const int np = (int)s->prims.size();
   if (np < kGridMinPrims) return TP_OK;
   bool moving = false;
@@ -684,9 +688,26 @@ tp_status upload_grid(tp_scene* s) {
       all.insert(all.end(), items.begin(), items.end());
       TP_CUDA(cudaMalloc(&s->d_grid, all.size() * sizeof(int)));
       TP_CUDA(cudaMemcpy(s->d_grid, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice));
+      s->grid_items = std::move(items);
     }
   }
   s->grid_cells = (int)ncell;
+  return TP_OK;
+}
+
+// The bounding spheres of the grid's items, from the primitive records of the
+// scene tables (the walk and the records then hold the same numbers).
+template <typename R>
+tp_status upload_grid_rows(tp_scene* s, const std::vector<uint8_t>& blob) {
+  if (s->grid_cells == 0) return TP_OK;
+  const auto* P = reinterpret_cast<const DPrim<R>*>(blob.data() + s->off_prims);
+  std::vector<GridRow<R>> rows(s->grid_items.size() + kGridChunk, GridRow<R>{});
+  for (size_t k = 0; k < s->grid_items.size(); ++k) {
+    const DPrim<R>& p = P[s->grid_items[k]];
+    rows[k] = GridRow<R>{{p.c[0], p.c[1], p.c[2]}, p.bound_r};
+  }
+  TP_CUDA(cudaMalloc(&s->d_grid_rows, rows.size() * sizeof(GridRow<R>)));
+  TP_CUDA(cudaMemcpy(s->d_grid_rows, rows.data(), rows.size() * sizeof(GridRow<R>), cudaMemcpyHostToDevice));
   return TP_OK;
 }
 
@@ -694,6 +715,8 @@ tp_status upload_blob(tp_scene* s) {
   tp_status gst = upload_grid(s);
   if (gst != TP_OK) return gst;
   std::vector<uint8_t> blob = s->precision == TP_FP64 ? build_blob<double>(s) : build_blob<float>(s);
+  gst = s->precision == TP_FP64 ? upload_grid_rows<double>(s, blob) : upload_grid_rows<float>(s, blob);
+  if (gst != TP_OK) return gst;
   if (blob.size() > s->blob_cap) {
     if (s->d_blob) cudaFree(s->d_blob);
     s->d_blob = nullptr;
@@ -766,6 +789,7 @@ void fill_common(const tp_scene* s, KParams<R>& k) {
   }
   k.grid_start = s->d_grid;
   k.grid_items = s->d_grid ? s->d_grid + s->grid_cells + 1 : nullptr;
+  k.grid_rows = static_cast<const GridRow<R>*>(s->d_grid_rows);
   k.n_inst = s->n_inst;
   k.inst_prefix = s->d_prefix;
   k.inst_first = s->d_first;
@@ -1612,7 +1636,7 @@ void tp_destroy_scene(tp_scene* s) {
   if (s->graph) cudaGraphExecDestroy(s->graph);
   if (s->capture_stream) cudaStreamDestroy(s->capture_stream);
   cudaFree(s->d_blob);
-  cudaFree(s->d_grid);
+  cudaFree(s->d_grid); cudaFree(s->d_grid_rows);
   cudaFree(s->d_sum); cudaFree(s->d_sumsq); cudaFree(s->d_J); cudaFree(s->d_J2);
   cudaFree(s->d_prefix); cudaFree(s->d_first); cudaFree(s->d_params); cudaFree(s->d_aux);
   cudaFree(s->d_work); cudaFree(s->d_counters); cudaFree(s->d_status);

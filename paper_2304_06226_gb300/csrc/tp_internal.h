@@ -73,6 +73,17 @@ struct alignas(16) DTally {
   int kind, trigger, volume, face, scat, nb0, nb1, offset;
 };
 
+// One entry of a grid cell's list: the bounding sphere of the primitive (its
+// centre and DPrim::bound_r), so that the walk reads the spheres of a cell from
+// consecutive rows.
+template <typename R>
+struct alignas(4 * sizeof(R)) GridRow {
+  R c[3], r;
+};
+// Rows the grid walk looks at in one round; the rows array has as many rows of
+// padding after the last item.
+constexpr int kGridChunk = 4;
+
 // Everything a transport launch needs.  The scene tables live in one blob in
 // global memory (16-byte aligned sections) that each CTA stages into shared
 // memory with a bulk asynchronous copy when it fits.
@@ -103,6 +114,7 @@ struct KParams {
   R grid_lo[3], grid_hi[3], grid_cell[3], grid_inv[3];
   const int* grid_start;
   const int* grid_items;
+  const GridRow<R>* grid_rows;   // beside each item, its bounding sphere
   // random numbers
   uint32_t key0, key1;
   int event_cap;
