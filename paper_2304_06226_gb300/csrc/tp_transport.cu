@@ -97,6 +97,8 @@ template <> struct Tr<float> {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
   }
+  // cos and sin of the azimuth 2 pi xi
+  static __device__ __forceinline__ void azimuth(float xi, float* sp, float* cp) { sincosf(kTwoPi * xi, sp, cp); }
   // Sums of products below name the product that is rounded by itself, so that
   // a neutron's path does not depend on what the compiler contracts where:
   // every kernel and build gives the same path bit for bit.
@@ -109,11 +111,13 @@ template <> struct Tr<float> {
 };
 template <> struct Tr<double> {
   static __device__ __forceinline__ double u01(uint32_t a) {
-    return ((double)a + 0.5) * 2.3283064365386963e-10;  // (a + 1/2) 2^-32
+    // (a + 1/2) 2^-32, exactly: 1 + a 2^-32 from its bits, less 1 - 2^-33
+    return __hiloint2double((int)(0x3FF00000u | (a >> 12)), (int)(a << 20)) - (1.0 - 1.1641532182693481e-10);
   }
-  static __device__ __forceinline__ double nudge(double m) { return 1e-9 * fmax(1.0, m); }
   static __device__ __forceinline__ double neg_log_u01(uint32_t a) { return -log(u01(a)); }
   static __device__ __forceinline__ double inf() { return __longlong_as_double(0x7ff0000000000000ll); }
+  // (the argument reduction of sincospi is a subtraction)
+  static __device__ __forceinline__ void azimuth(double xi, double* sp, double* cp) { sincospi(2.0 * xi, sp, cp); }
   static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
   static __device__ __forceinline__ double root(double x) { return sqrt(x); }
   static __device__ __forceinline__ double rroot(double x) { return 1.0 / sqrt(x); }
@@ -456,10 +460,23 @@ __device__ R exit_dist(const DPrim<R>& p, R dR, const R x[3], const R u[3], int*
   R best = Tr<R>::inf();
   int bf = -1;
   if (p.shape == TP_BOX) {
+    if constexpr (sizeof(R) == 8) {
+      // the nearest of the three faces by cross-multiplication, one division
+      // (three reciprocals were a third of the FP64 instructions of a slab's flight)
+      R bn = R(1), bd = R(0);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const R t = Tr<R>::quot(copysign(p.p[a], v[a]) - q[a], Tr<R>::rcp(v[a]));
-      if (v[a] != R(0) && t < best) { best = t; bf = 2 * a + (v[a] > R(0) ? 1 : 0); }
+      for (int a = 0; a < 3; ++a) {
+        const bool neg = signbit(v[a]);
+        const R n = p.p[a] + (neg ? q[a] : -q[a]), d = fabs(v[a]);
+        if (n * bd < bn * d) { bn = n; bd = d; bf = 2 * a + (neg ? 0 : 1); }
+      }
+      best = bf >= 0 ? bn / bd : best;
+    } else {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const R t = Tr<R>::quot(copysign(p.p[a], v[a]) - q[a], Tr<R>::rcp(v[a]));
+        if (v[a] != R(0) && t < best) { best = t; bf = 2 * a + (v[a] > R(0) ? 1 : 0); }
+      }
     }
   } else {
     const bool tube = p.shape == TP_TUBE;
@@ -643,12 +660,12 @@ __device__ __forceinline__ void normal(const DPrim<R>& p, const R x[3], int face
   n[0] = d[0] * inv; n[1] = d[1] * inv; n[2] = d[2] * inv;
 }
 
-// Deflection by polar cosine mu and azimuth phi about u.
+// Deflection by polar cosine mu and azimuth 2 pi xphi about u.
 template <typename R>
-__device__ __forceinline__ void rotate(R u[3], R mu, R phi) {
+__device__ __forceinline__ void rotate(R u[3], R mu, R xphi) {
   const R st = Tr<R>::root(fmax(R(0), Tr<R>::fma(-mu, mu, R(1))));
   R sp, cp;
-  d_sincos(phi, &sp, &cp);
+  Tr<R>::azimuth(xphi, &sp, &cp);
   const R t2 = Tr<R>::fma(-u[2], u[2], R(1));
   R o0, o1, o2;
   if (t2 > R(1e-20)) {
@@ -733,6 +750,27 @@ __device__ __forceinline__ int bin1(R x, R lo, R hi, R inv_w, int n) {
   return (b >= 0 && b < n) ? b : (b >= n ? n - 1 : -1);
 }
 
+// Bin of the angle between (x - origin) and the tally axis.  FP64: an FP32 angle
+// (good to 2e-6 rad) settles the bin unless it lies that near a bin's edge; then,
+// and only then, the FP64 angle is taken, so the bin is always the FP64 one.
+template <typename R>
+__device__ __forceinline__ R tally_angle(const DTally<R>& T, R x0, R x1, R x2);
+
+template <typename R>
+__device__ __forceinline__ int angle_bin(const DTally<R>& T, R x0, R x1, R x2) {
+  if constexpr (sizeof(R) == 8) {
+    const float v0 = (float)(x0 - T.origin[0]), v1 = (float)(x1 - T.origin[1]), v2 = (float)(x2 - T.origin[2]);
+    const float a0 = (float)T.axis[0], a1 = (float)T.axis[1], a2 = (float)T.axis[2];
+    const float c0 = v1 * a2 - v2 * a1, c1 = v2 * a0 - v0 * a2, c2 = v0 * a1 - v1 * a0;
+    const float th = atan2f(sqrtf(c0 * c0 + c1 * c1 + c2 * c2), v0 * a0 + v1 * a1 + v2 * a2);
+    const float w = (float)T.inv_w[0];
+    const float y = (th - (float)T.lo[0]) * w, slack = 4e-6f * w + 1e-6f * (float)T.nb0;
+    const float b = floorf(y);
+    if (y - b > slack && b + 1.0f - y > slack && b >= 0.0f && b < (float)T.nb0) return (int)b;
+  }
+  return bin1(tally_angle(T, x0, x1, x2), T.lo[0], T.hi[0], T.inv_w[0], T.nb0);
+}
+
 // angle between (x - origin) and the tally axis, accurate at small angles
 template <typename R>
 __device__ __forceinline__ R tally_angle(const DTally<R>& T, R x0, R x1, R x2) {
@@ -748,7 +786,7 @@ __device__ __forceinline__ int tally_bin(const DTally<R>& T, R x0, R x1, R x2, R
   if constexpr (!(OPT & kOptFull)) {
     // lean build: count, angular and PSD scorers only
     if (T.kind == TP_TALLY_COUNT) return 0;
-    if (T.kind == TP_TALLY_ANGULAR) return bin1(tally_angle(T, x0, x1, x2), T.lo[0], T.hi[0], T.inv_w[0], T.nb0);
+    if (T.kind == TP_TALLY_ANGULAR) return angle_bin(T, x0, x1, x2);
     const int bx = bin1(x0, T.lo[0], T.hi[0], T.inv_w[0], T.nb0);
     const int by = bin1(x1, T.lo[1], T.hi[1], T.inv_w[1], T.nb1);
     return (bx < 0 || by < 0) ? -1 : bx * T.nb1 + by;
@@ -756,7 +794,7 @@ __device__ __forceinline__ int tally_bin(const DTally<R>& T, R x0, R x1, R x2, R
     switch (T.kind) {
       case TP_TALLY_COUNT: return 0;
       case TP_TALLY_TOF: return bin1(path * lam * R(1.0 / kHoverMn), T.lo[0], T.hi[0], T.inv_w[0], T.nb0);
-      case TP_TALLY_ANGULAR: return bin1(tally_angle(T, x0, x1, x2), T.lo[0], T.hi[0], T.inv_w[0], T.nb0);
+      case TP_TALLY_ANGULAR: return angle_bin(T, x0, x1, x2);
       case TP_TALLY_MULTISCAT: return bin1((R)nscat, T.lo[0], T.hi[0], T.inv_w[0], T.nb0);
       case TP_TALLY_DQ: {
         // elastic momentum transfer Q = 4 pi sin(theta/2) / lambda (Eq. eQelastic)
@@ -908,7 +946,16 @@ __device__ bool source(const KParams<R>& kp, const View<R>& V, Particle<R>& P, R
 
 template <typename R>
 __device__ __forceinline__ R nudge_len(const R x[3]) {
-  return Tr<R>::nudge(fmax(fabs(x[0]), fmax(fabs(x[1]), fabs(x[2]))));
+  if constexpr (sizeof(R) == 8) {
+    // the largest magnitude by its bits: integer comparisons instead of three
+    // on the FP64 pipe, which bounds the FP64 kernels
+    constexpr long long kOne = 0x3ff0000000000000ll;
+    const long long a = __double_as_longlong(fabs(x[0])), b = __double_as_longlong(fabs(x[1])),
+                    c = __double_as_longlong(fabs(x[2]));
+    return 1e-9 * __longlong_as_double(max(max(a, b), max(c, kOne)));
+  } else {
+    return Tr<R>::nudge(fmax(fabs(x[0]), fmax(fabs(x[1]), fabs(x[2]))));
+  }
 }
 
 // Draw the new direction of a scatter by process `proc` of material `mat`.
@@ -919,7 +966,7 @@ __device__ __forceinline__ void scatter_dir(const View<R>& V, int mat, int proc,
     const R mu = R(2) * xmu - R(1);
     const R st = Tr<R>::root(fmax(R(0), Tr<R>::fma(-mu, mu, R(1))));
     R sp, cp;
-    d_sincos(Tr<R>::kTwoPi * xphi, &sp, &cp);
+    Tr<R>::azimuth(xphi, &sp, &cp);
     u[0] = st * cp; u[1] = st * sp; u[2] = mu;
   } else {
     const DMat<R>& m = V.mats[mat];
@@ -933,7 +980,7 @@ __device__ __forceinline__ void scatter_dir(const View<R>& V, int mat, int proc,
       if (target < cum[mid + 1]) hi = mid; else lo = mid + 1;
     }
     const R sb = Tr<R>::quot(lam, Tr<R>::rcp(R(2) * V.line_d[m.line_off + lo]));
-    rotate(u, Tr<R>::fma(R(-2) * sb, sb, R(1)), Tr<R>::kTwoPi * xphi);
+    rotate(u, Tr<R>::fma(R(-2) * sb, sb, R(1)), xphi);
   }
 }
 
@@ -1029,11 +1076,21 @@ __device__ __forceinline__ void entry_test(const View<R>& V, R dR, const R x[3],
   const DPrim<R>& pi = V.prims[i];
   if (i == last && last_hull) return;
   // bounding sphere: skip if the ray misses it or moves away from outside it
-  const R q0 = x[0] - pi.c[0], q1 = x[1] - pi.c[1], q2 = x[2] - pi.c[2];
-  const R qu = dot3(q0, u[0], q1, u[1], q2, u[2]);
-  const R qq = dot3(q0, q0, q1, q1, q2, q2);
-  const R rb2 = pi.bound_r * pi.bound_r;
-  if (qq > rb2 && (qu >= R(0) || Tr<R>::fma(-qu, qu, qq) > rb2)) return;
+  if constexpr (sizeof(R) == 8) {
+    // in FP32 with room for its rounding (a part in 1e4 of the distance): who
+    // passes is settled by the FP64 entry distance
+    const float q0 = (float)(x[0] - pi.c[0]), q1 = (float)(x[1] - pi.c[1]), q2 = (float)(x[2] - pi.c[2]);
+    const float w0 = (float)u[0], w1 = (float)u[1], w2 = (float)u[2], r = (float)pi.bound_r;
+    const float qu = q0 * w0 + q1 * w1 + q2 * w2, qq = q0 * q0 + q1 * q1 + q2 * q2;
+    const float rb2 = r * r + 1e-4f * (qq + r * r);
+    if (qq > rb2 && (qu * qu * (qu >= 0.0f ? 0.0f : 1.0f) < qq - rb2)) return;
+  } else {
+    const R q0 = x[0] - pi.c[0], q1 = x[1] - pi.c[1], q2 = x[2] - pi.c[2];
+    const R qu = dot3(q0, u[0], q1, u[1], q2, u[2]);
+    const R qq = dot3(q0, q0, q1, q1, q2, q2);
+    const R rb2 = pi.bound_r * pi.bound_r;
+    if (qq > rb2 && (qu >= R(0) || Tr<R>::fma(-qu, qu, qq) > rb2)) return;
+  }
   int f;
   const R t = entry_dist(pi, dR, x, u, &f, i == last ? tmin : R(0));
   if (t < *db) { *db = t; *target = i; *face = f; }
