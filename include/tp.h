@@ -251,8 +251,8 @@ typedef struct {
  *   threads) selects the 64-register one.  kernel 0 lets the autotuner pick
  *   the variant, block size, build and table staging on the scene's first run
  *   (with and without gradients separately).
- * use_graph: 1 = run as a CUDA graph [work-description copies, work-counter
- *   reset, persistent kernel] captured on the first call with a given launch
+ * use_graph: 1 = run as a CUDA graph [work-description copy (with the work
+ *   counter at 0), persistent kernel] captured on the first call with a given launch
  *   (kernel, block, CTAs, gradients, seed, total histories, records) and
  *   replayed afterwards; history counts and first ids may change between
  *   replays (they are read from the scene's pinned staging buffer).

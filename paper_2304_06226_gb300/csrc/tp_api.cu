@@ -155,7 +155,8 @@ struct tp_scene {
   double *d_sum = nullptr, *d_sumsq = nullptr, *d_J = nullptr, *d_J2 = nullptr;
   std::vector<double> n_done;  // histories run per instance
   // per-run work description
-  unsigned long long *d_prefix = nullptr, *d_first = nullptr, *h_stage = nullptr;
+  unsigned long long *d_prefix = nullptr, *d_first = nullptr, *h_stage = nullptr;   // (after the work counter)
+  size_t clear_bytes = 0;   // the block of tallies, counters and status, from d_sum
   void* d_params = nullptr;   // instance parameters in the transport precision
   double* d_aux = nullptr;  // backward: [n_inst][n_par] scale + [n_inst] n_done
   double* h_aux = nullptr;
@@ -171,6 +172,8 @@ struct tp_scene {
   // launch configuration: last used, and the autotuned choice per gradient mode
   int kernel = 0, block = 0, ctas_per_sm = 0;
   LaunchCfg last_cfg{};   // the last run's complete configuration
+  LaunchCfg resolved{};   // what resolve() last worked out, and from what
+  int resolved_key[11] = {};
   int launches = 0;   // transport kernels of the last run
   int smem_optin = 0; // shared memory a block may use on this device (queried once)
   int tuned_kernel[2] = {0, 0}, tuned_block[2] = {0, 0}, tuned_stage[2] = {-1, -1}, tuned_hi[2] = {-1, -1};
@@ -188,6 +191,9 @@ struct tp_scene {
 };
 
 namespace {
+
+// Words of a run's description: the work counter (0), prefix sums, first ids.
+size_t work_words(const tp_scene* s) { return 2 + 2 * (size_t)s->n_inst; }
 
 // ---------------------------------------------------------------------------
 // Validation helpers
@@ -855,6 +861,15 @@ tp_status resolve(tp_scene* s, bool grad, int kernel, int req_block, int req_cta
   const int b = req_block > 0 ? req_block : 256;
   if (b % 32 != 0 || b < 32 || b > 256)
     return fail(TP_ERR_INVALID_ARG, "kernel %d block_size %d: need a multiple of 32 in [32, 256]", kernel, b);
+  // the last answer, while what it was worked out from is the same (the
+  // occupancy queries take as long as a small run's launch)
+  const int key[] = {grad, kernel, b, req_ctas, stage, hi, weighted, s->full, (int)s->blob_bytes, s->grid_cells > 0,
+                     counts_only(s)};
+  static_assert(sizeof key == sizeof s->resolved_key, "resolve key");
+  if (s->resolved.kernel != 0 && std::memcmp(key, s->resolved_key, sizeof key) == 0) {
+    *c = s->resolved;
+    return TP_OK;
+  }
   if (s->smem_optin == 0) {
     int dev = 0;
     TP_CUDA(cudaGetDevice(&dev));
@@ -882,6 +897,8 @@ tp_status resolve(tp_scene* s, bool grad, int kernel, int req_block, int req_cta
   }
   if (occ < 1) return fail(TP_ERR_INVALID_ARG, "kernel %d block_size %d does not fit on an SM", kernel, b);
   *c = LaunchCfg{kernel, b, req_ctas > 0 ? std::min(req_ctas, occ) : occ, stage, h, 0, s->full, 1, count};
+  s->resolved = *c;
+  std::memcpy(s->resolved_key, key, sizeof key);
   return TP_OK;
 }
 
@@ -895,7 +912,7 @@ struct Outputs {
 template <typename R>
 cudaError_t launch_one(tp_scene* s, const LaunchCfg& c, bool grad, uint64_t seed, unsigned long long total,
                        tp_record* records, unsigned long long n_records, const Outputs& o, cudaStream_t st,
-                       int sec_mode = 0, unsigned long long index_base = 0) {
+                       int sec_mode = 0, unsigned long long index_base = 0, bool first = false) {
   KParams<R> k{};
   fill_common(s, k);
   k.sec_mode = sec_mode;
@@ -914,7 +931,8 @@ cudaError_t launch_one(tp_scene* s, const LaunchCfg& c, bool grad, uint64_t seed
   const int grid = s->sm_count * c.ctas;
   const long long warps = (long long)grid * (c.block / 32);
   k.chunk = sec_mode == 2 ? 16 : (int)std::max(1ll, std::min(256ll, (long long)(total / (unsigned long long)(warps * 8))));
-  cudaError_t e = cudaMemsetAsync(s->d_work, 0, sizeof(unsigned long long), st);
+  // the first launch after the run's description finds the counter at 0
+  cudaError_t e = first ? cudaSuccess : cudaMemsetAsync(s->d_work, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   const size_t sm = smem_variant(s, c.variant(), grad, c.block, c.stage);
   if constexpr (std::is_same<R, double>::value) return launch_transport_f64(k, c.variant(), grad, grid, c.block, sm, st);
@@ -961,15 +979,15 @@ tp_status ensure_sec(tp_scene* s, unsigned long long total) {
 // second pass of the plain warp-pool kernel over the queue.
 template <typename R>
 cudaError_t launch_run(tp_scene* s, const LaunchCfg& c, bool grad, uint64_t seed, unsigned long long total,
-                       tp_record* records, unsigned long long n_records, const Outputs& o, cudaStream_t st) {
-  if (!grad || !c.defer) return launch_one<R>(s, c, grad, seed, total, records, n_records, o, st);
+                       tp_record* records, unsigned long long n_records, const Outputs& o, cudaStream_t st, bool first) {
+  if (!grad || !c.defer) return launch_one<R>(s, c, grad, seed, total, records, n_records, o, st, 0, 0, first);
   if (!s->d_sec || s->sec_cfg.kernel == 0) return cudaErrorInvalidValue;   // ensure_sec comes first
   const LaunchCfg& sc = s->sec_cfg;
   const unsigned long long chunk = std::max(1ull, s->sec_cap / kSecPerHistory);
   for (unsigned long long c0 = 0; c0 < total; c0 += chunk) {
     const unsigned long long n = std::min(chunk, total - c0);
     cudaError_t e = cudaMemsetAsync(s->d_sec_count, 0, sizeof(unsigned long long), st);
-    if (e == cudaSuccess) e = launch_one<R>(s, c, true, seed, n, records, n_records, o, st, 1, c0);
+    if (e == cudaSuccess) e = launch_one<R>(s, c, true, seed, n, records, n_records, o, st, 1, c0, first && c0 == 0);
     if (e == cudaSuccess) e = launch_one<R>(s, sc, false, seed, 0, nullptr, 0, o, st, 2, 0);
     if (e != cudaSuccess) return e;
   }
@@ -977,9 +995,10 @@ cudaError_t launch_run(tp_scene* s, const LaunchCfg& c, bool grad, uint64_t seed
 }
 
 cudaError_t launch_cfg(tp_scene* s, const LaunchCfg& c, bool grad, uint64_t seed, unsigned long long total,
-                       tp_record* records, unsigned long long n_records, const Outputs& o, cudaStream_t st) {
-  if (s->precision == TP_FP64) return launch_run<double>(s, c, grad, seed, total, records, n_records, o, st);
-  return launch_run<float>(s, c, grad, seed, total, records, n_records, o, st);
+                       tp_record* records, unsigned long long n_records, const Outputs& o, cudaStream_t st,
+                       bool first = false) {
+  if (s->precision == TP_FP64) return launch_run<double>(s, c, grad, seed, total, records, n_records, o, st, first);
+  return launch_run<float>(s, c, grad, seed, total, records, n_records, o, st, first);
 }
 
 // Times every candidate (kernel, block size) on up to 2^22 of this run's
@@ -1066,9 +1085,9 @@ tp_status autotune(tp_scene* s, bool grad, uint64_t seed, unsigned long long tot
   return TP_OK;
 }
 
-// Runs [work-description copies, work-counter reset, kernel] as a CUDA graph,
+// Runs [work-description copy (work counter included), kernel] as a CUDA graph,
 // captured on a private stream the first time a launch key is seen and
-// replayed on `st` afterwards.  The copies read the pinned staging buffer at
+// replayed on `st` afterwards.  The copy reads the pinned staging buffer at
 // replay time, so counts and first ids may change between replays.
 tp_status run_graph(tp_scene* s, const LaunchCfg& cfg, bool grad, const tp_run* r, unsigned long long total,
                     const Outputs& o, cudaStream_t st) {
@@ -1082,12 +1101,9 @@ tp_status run_graph(tp_scene* s, const LaunchCfg& cfg, bool grad, const tp_run* 
     if (!s->capture_stream) TP_CUDA(cudaStreamCreateWithFlags(&s->capture_stream, cudaStreamNonBlocking));
     cudaStream_t cs = s->capture_stream;
     TP_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    cudaError_t ce = cudaMemcpyAsync(s->d_prefix, s->h_stage, (s->n_inst + 1) * sizeof(unsigned long long),
+    cudaError_t ce = cudaMemcpyAsync(s->d_work, s->h_stage, work_words(s) * sizeof(unsigned long long),
                                      cudaMemcpyHostToDevice, cs);
-    if (ce == cudaSuccess)
-      ce = cudaMemcpyAsync(s->d_first, s->h_stage + s->n_inst + 1, s->n_inst * sizeof(unsigned long long),
-                           cudaMemcpyHostToDevice, cs);
-    if (ce == cudaSuccess) ce = launch_cfg(s, cfg, grad, r->seed, total, r->records, r->n_records, o, cs);
+    if (ce == cudaSuccess) ce = launch_cfg(s, cfg, grad, r->seed, total, r->records, r->n_records, o, cs, true);
     cudaGraph_t g = nullptr;
     const cudaError_t ee = cudaStreamEndCapture(cs, &g);
     if (ce == cudaSuccess) ce = ee;
@@ -1253,21 +1269,25 @@ tp_status tp_create_scene(const tp_scene_desc* d, tp_scene** out) {
     if (r != cudaSuccess) { fail(r == cudaErrorMemoryAllocation ? TP_ERR_OOM : TP_ERR_CUDA, "cudaMalloc(%zu): %s", bytes, cudaGetErrorString(r)); return false; }
     return true;
   };
-  if (!alloc((void**)&s->d_sum, nb * sizeof(double)) || !alloc((void**)&s->d_sumsq, nb * sizeof(double)))
-    return bail(TP_ERR_OOM);
+  // sum, sumsq, J, J2, counters and status in one block: a reset is one memset
+  const size_t arrays = 2 + 2 * (size_t)s->n_par;
+  s->clear_bytes = arrays * nb * sizeof(double) + (kNumCounters + 1) * sizeof(unsigned long long);
+  if (!alloc((void**)&s->d_sum, s->clear_bytes)) return bail(TP_ERR_OOM);
+  s->d_sumsq = s->d_sum + nb;
   if (s->n_par > 0) {
-    if (!alloc((void**)&s->d_J, nb * s->n_par * sizeof(double)) || !alloc((void**)&s->d_J2, nb * s->n_par * sizeof(double)))
-      return bail(TP_ERR_OOM);
+    s->d_J = s->d_sumsq + nb;
+    s->d_J2 = s->d_J + nb * s->n_par;
   }
-  if (!alloc((void**)&s->d_prefix, (s->n_inst + 1) * sizeof(unsigned long long)) ||
-      !alloc((void**)&s->d_first, s->n_inst * sizeof(unsigned long long)) ||
-      !alloc((void**)&s->d_params, (size_t)s->n_inst * kMaxPar * sizeof(double)) ||
-      !alloc((void**)&s->d_aux, ((size_t)s->n_inst * (kMaxPar + 1)) * sizeof(double)) ||
-      !alloc((void**)&s->d_work, sizeof(unsigned long long)) ||
-      !alloc((void**)&s->d_counters, kNumCounters * sizeof(unsigned long long)) ||
-      !alloc((void**)&s->d_status, sizeof(int)))
+  s->d_counters = reinterpret_cast<unsigned long long*>(s->d_sum + arrays * nb);
+  s->d_status = reinterpret_cast<int*>(s->d_counters + kNumCounters);
+  // work counter, prefix sums and first ids in one block: a run's description is one copy
+  if (!alloc((void**)&s->d_work, work_words(s) * sizeof(unsigned long long))) return bail(TP_ERR_OOM);
+  s->d_prefix = s->d_work + 1;
+  s->d_first = s->d_prefix + (s->n_inst + 1);
+  if (!alloc((void**)&s->d_params, (size_t)s->n_inst * kMaxPar * sizeof(double)) ||
+      !alloc((void**)&s->d_aux, ((size_t)s->n_inst * (kMaxPar + 1)) * sizeof(double)))
     return bail(TP_ERR_OOM);
-  if (cudaMallocHost((void**)&s->h_stage, (2 * (size_t)s->n_inst + 1) * sizeof(unsigned long long)) != cudaSuccess ||
+  if (cudaMallocHost((void**)&s->h_stage, work_words(s) * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMallocHost((void**)&s->h_aux, ((size_t)s->n_inst * (kMaxPar + 1)) * sizeof(double)) != cudaSuccess)
     return bail(fail(TP_ERR_OOM, "pinned staging buffers"));
   if (cudaEventCreateWithFlags(&s->stage_done, cudaEventDisableTiming) != cudaSuccess)
@@ -1352,15 +1372,23 @@ tp_status tp_set_params(tp_scene* s, const double* inst_params) {
       }
       s->inst_params[(size_t)q * kMaxPar + p] = v;
     }
-  tp_status st = validate_geometry(s);
-  if (st != TP_OK) {
-    s->inst_params = old;
-    return st;
+  // Only a primitive bound to the radius moves with the parameters: without one
+  // the geometry, its checks and its tables stay as they are (on the
+  // 1000-primitive scene checking pairs and rebuilding tables and grid is 2 ms
+  // a fit step, a tenth of the step's run).
+  bool moving = false;
+  for (const auto& p : s->prims) moving |= (p.bind_rmin || p.bind_rmax);
+  if (moving) {
+    tp_status st = validate_geometry(s);
+    if (st != TP_OK) {
+      s->inst_params = old;
+      return st;
+    }
   }
   TP_CUDA(cudaDeviceSynchronize());
   const std::vector<uint8_t> pb = params_bytes(s->inst_params, s->precision);
   TP_CUDA(cudaMemcpy(s->d_params, pb.data(), pb.size(), cudaMemcpyHostToDevice));
-  s->blob_dirty = true;   // bounding radii and neighbour lists depend on the radii
+  if (moving) s->blob_dirty = true;   // bounding radii and neighbour lists depend on the radii
   return TP_OK;
 }
 
@@ -1369,15 +1397,7 @@ tp_status tp_reset_tallies(tp_scene* s) {
   // a run still draining after tp_abort must have stopped before the flag clears
   TP_CUDA(cudaDeviceSynchronize());
   if (s->h_abort) *s->h_abort = 0;
-  const size_t nb = (size_t)s->n_inst * std::max(1, s->total_bins);
-  TP_CUDA(cudaMemset(s->d_sum, 0, nb * sizeof(double)));
-  TP_CUDA(cudaMemset(s->d_sumsq, 0, nb * sizeof(double)));
-  if (s->d_J) {
-    TP_CUDA(cudaMemset(s->d_J, 0, nb * s->n_par * sizeof(double)));
-    TP_CUDA(cudaMemset(s->d_J2, 0, nb * s->n_par * sizeof(double)));
-  }
-  TP_CUDA(cudaMemset(s->d_counters, 0, kNumCounters * sizeof(unsigned long long)));
-  TP_CUDA(cudaMemset(s->d_status, 0, sizeof(int)));
+  TP_CUDA(cudaMemset(s->d_sum, 0, s->clear_bytes));   // tallies, counters and status are one block
   std::fill(s->n_done.begin(), s->n_done.end(), 0.0);
   return TP_OK;
 }
@@ -1404,11 +1424,12 @@ tp_status tp_run_histories(tp_scene* s, const tp_run* r) {
     const unsigned long long first = r->first_history ? r->first_history[i] : 0ull;
     if (r->n_histories[i] > 0xffffffffull || first > 0x100000000ull - r->n_histories[i])
       return fail(TP_ERR_INVALID_ARG, "instance %d: history ids must stay below 2^32", i);
-    s->h_stage[i] = total;
-    s->h_stage[s->n_inst + 1 + i] = first;
+    s->h_stage[1 + i] = total;
+    s->h_stage[s->n_inst + 2 + i] = first;
     total += r->n_histories[i];
   }
-  s->h_stage[s->n_inst] = total;
+  s->h_stage[0] = 0;   // the work counter
+  s->h_stage[1 + s->n_inst] = total;
   if (total == 0) return TP_OK;
   if (r->secondaries < 0 || r->secondaries > 2) return fail(TP_ERR_INVALID_ARG, "secondaries %d", r->secondaries);
   if (r->stage < 0 || r->stage > 2) return fail(TP_ERR_INVALID_ARG, "stage %d: need 0, 1 or 2", r->stage);
@@ -1423,8 +1444,7 @@ tp_status tp_run_histories(tp_scene* s, const tp_run* r) {
   if (kernel == TP_KERNEL_AUTO) {
     if (s->tuned_kernel[grad] == 0) {
       // the trials read this run's work description
-      TP_CUDA(cudaMemcpyAsync(s->d_prefix, s->h_stage, (s->n_inst + 1) * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
-      TP_CUDA(cudaMemcpyAsync(s->d_first, s->h_stage + s->n_inst + 1, s->n_inst * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
+      TP_CUDA(cudaMemcpyAsync(s->d_work, s->h_stage, work_words(s) * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
       tp_status e = autotune(s, grad, r->seed, total, st);
       if (e != TP_OK) return e;
       if (grad && !s->tuned_defer && r->secondaries != 2 && s->d_sec) {   // not needed: give it back
@@ -1450,11 +1470,10 @@ tp_status tp_run_histories(tp_scene* s, const tp_run* r) {
     e = run_graph(s, cfg, grad, r, total, o, st);
     if (e != TP_OK) return e;
   } else {
-    TP_CUDA(cudaMemcpyAsync(s->d_prefix, s->h_stage, (s->n_inst + 1) * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
-    TP_CUDA(cudaMemcpyAsync(s->d_first, s->h_stage + s->n_inst + 1, s->n_inst * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
+    TP_CUDA(cudaMemcpyAsync(s->d_work, s->h_stage, work_words(s) * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
     TP_CUDA(cudaEventRecord(s->stage_done, st));
     s->stage_pending = true;
-    cudaError_t ce = launch_cfg(s, cfg, grad, r->seed, total, r->records, r->n_records, o, st);
+    cudaError_t ce = launch_cfg(s, cfg, grad, r->seed, total, r->records, r->n_records, o, st, true);
     if (ce != cudaSuccess) return fail(TP_ERR_CUDA, "transport launch: %s", cudaGetErrorString(ce));
   }
   for (int i = 0; i < s->n_inst; ++i) s->n_done[i] += (double)r->n_histories[i];
@@ -1637,9 +1656,9 @@ void tp_destroy_scene(tp_scene* s) {
   if (s->capture_stream) cudaStreamDestroy(s->capture_stream);
   cudaFree(s->d_blob);
   cudaFree(s->d_grid); cudaFree(s->d_grid_rows);
-  cudaFree(s->d_sum); cudaFree(s->d_sumsq); cudaFree(s->d_J); cudaFree(s->d_J2);
-  cudaFree(s->d_prefix); cudaFree(s->d_first); cudaFree(s->d_params); cudaFree(s->d_aux);
-  cudaFree(s->d_work); cudaFree(s->d_counters); cudaFree(s->d_status);
+  cudaFree(s->d_sum);    // with sumsq, J, J2, counters and status
+  cudaFree(s->d_work);   // with the prefix sums and first ids
+  cudaFree(s->d_params); cudaFree(s->d_aux);
   cudaFree(s->d_sec); cudaFree(s->d_sec_count);
   if (s->h_stage) cudaFreeHost(s->h_stage);
   if (s->h_aux) cudaFreeHost(s->h_aux);

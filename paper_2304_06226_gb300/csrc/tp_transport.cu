@@ -23,6 +23,7 @@
 // independent of the launch shape and of which lane ran which history.
 //
 // Tallies are FP64 sums of w and w^2 per bin (plus the score-function tallies),
+// counted in shared memory where every weight is 1 (see score), else
 // added with warp-aggregated atomics: the lanes hitting one bin find each other
 // once per score, sum their values by pointer jumping over their group
 // (shuffles, in the transport precision) and the group's lowest lane issues one
