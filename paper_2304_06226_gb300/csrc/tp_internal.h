@@ -125,7 +125,7 @@ struct KParams {
   const R* inst_params;                   // [n_inst][kMaxPar], device, transport precision
   unsigned long long total;
   unsigned long long* work_counter;
-  int chunk;  // histories a warp claims at once
+  int chunk;  // history kernel: histories a warp claims at once
   // event kernel, plain runs: the bank is regrouped every `regroup` events
   // (1 = every event); in between, each thread continues its own neutron
   int regroup;
