@@ -718,6 +718,13 @@ tp_status upload_grid_rows(tp_scene* s, const std::vector<uint8_t>& blob) {
 }
 
 tp_status upload_blob(tp_scene* s) {
+  // A captured graph has the tables' addresses, section offsets, grid and
+  // geometry flags baked in: new tables end it.
+  if (s->graph) {
+    if (s->stage_pending) { TP_CUDA(cudaEventSynchronize(s->stage_done)); s->stage_pending = false; }
+    cudaGraphExecDestroy(s->graph);
+    s->graph = nullptr;
+  }
   tp_status gst = upload_grid(s);
   if (gst != TP_OK) return gst;
   std::vector<uint8_t> blob = s->precision == TP_FP64 ? build_blob<double>(s) : build_blob<float>(s);
