@@ -2298,6 +2298,7 @@ __global__ void __launch_bounds__(256, MINB) k_transport_wq(const __grid_constan
       else to = pool_advance<R, GRAD, OPT>(kp, V, pool, slot, q == Q_ADVP, cnt);
     }
     // ---- push each slot to the stack of its next event ----
+    __syncwarp();   // every lane has popped: a push may reuse the entries above
     unsigned added = 0u, mine = 0u;
 #pragma unroll
     for (int k = 0; k < kNumQ; ++k) {

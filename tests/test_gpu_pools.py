@@ -43,6 +43,29 @@ def test_pool_steps(scene, n, block):
             assert np.allclose(got[k], v, rtol=1e-12, atol=1e-12 * max(1e-300, np.abs(v).max())), k
 
 
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+@pytest.mark.parametrize("scene", ["slab", "guide"])
+def test_every_history_runs_once_and_as_in_the_history_kernel(scene, precision):
+    """Slots return to the stacks a step popped them from.  A slot listed twice or
+    lost would end a history early, twice or never: each path is that of the
+    history kernel, word for word (the geometry is explicit arithmetic); the
+    weight, a product of at most a hundred factors, to their rounding."""
+    from paper_2304_06226_gb300.engine import Scene, new_records, records_to_numpy
+    n, out = 100_003, []
+    sc = Scene({"slab": lambda: W.slab(g=3.0, precision=precision), "guide": lambda: W.guide(precision=precision)}[scene]())
+    for kernel in (1, 3):
+        rec = new_records(n)
+        sc.run(n, kernel=kernel, records=rec)
+        torch.cuda.synchronize()
+        out.append(records_to_numpy(rec))
+    sc.close()
+    for k, v in out[0].items():
+        if k == "w_final":
+            assert np.allclose(out[1][k], v, rtol=100 * (2.0 ** -23 if precision == "f32" else 2.0 ** -52), atol=0.0)
+        else:
+            assert np.array_equal(out[1][k], v, equal_nan=v.dtype.kind == "f"), k
+
+
 # Scenes whose weights stay 1: the pools count in shared memory, the event
 # kernel adds w and w^2 with FP64 atomics; both are whole numbers and equal.
 # 4096 bins are the most a histogram holds; with one more the pools add weights.
