@@ -718,10 +718,12 @@ tp_status upload_grid_rows(tp_scene* s, const std::vector<uint8_t>& blob) {
 }
 
 tp_status upload_blob(tp_scene* s) {
+  // An earlier run may still read the tables, on a stream that the copies below
+  // do not wait for.
+  TP_CUDA(cudaDeviceSynchronize());
   // A captured graph has the tables' addresses, section offsets, grid and
   // geometry flags baked in: new tables end it.
   if (s->graph) {
-    if (s->stage_pending) { TP_CUDA(cudaEventSynchronize(s->stage_done)); s->stage_pending = false; }
     cudaGraphExecDestroy(s->graph);
     s->graph = nullptr;
   }

@@ -1,7 +1,8 @@
 """Runs of one scene before and after its materials, biases or parameters change,
 against a scene that had the new values from the start.  FP64 on the history
 kernel: every history has its own random numbers, so counters are equal and the
-tallies agree to the rounding of their sums (at most 2e4 FP64 additions: 1e-11)."""
+tallies agree to the rounding of their sums (up to 2e6 FP64 additions of like
+sign, whose errors add like a random walk: 1e-11)."""
 import copy
 
 import numpy as np
@@ -69,4 +70,30 @@ def test_graph_run_after_the_tables_changed(change):
     sc.run(N, kernel=1, graph=True)   # the same seed and counts as the first graph
     torch.cuda.synchronize()
     same(sc, fresh(new))
+    sc.close()
+
+
+@pytest.mark.parametrize("grid", [False, True])
+def test_tables_change_behind_a_run_in_flight_on_a_side_stream(grid):
+    """The first run is still on its way (some milliseconds) when the bias changes
+    and the second is queued behind it: each must see its own tables."""
+    from paper_2304_06226_gb300.engine import Scene
+    old = W.imaging(n_prims=60, precision="f64", psd_bins=16) if grid else W.slab(g=1.0)
+    m, n = len(old["materials"]), (400_000 if grid else 2_000_000)
+    sc = Scene(old)
+    seen = []
+    for stream in (None, torch.cuda.Stream()):
+        for k in range(m):
+            sc.set_bias(k, old["bias"][k])
+        sc.reset()
+        torch.cuda.synchronize()
+        sc.run(n, kernel=1, stream=stream)
+        if stream is None:
+            torch.cuda.synchronize()
+        for k in range(m):
+            sc.set_bias(k, (0.5, 3.0, 1.0))
+        sc.run(1000, first=n, kernel=1, stream=stream)
+        torch.cuda.synchronize()
+        seen.append((sc.raw(), sc.counters()))
+    same(sc, seen[0])
     sc.close()
