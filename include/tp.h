@@ -24,6 +24,9 @@
  *    `on_device` flag of the call says.
  *  - GPU work is ordered on the CUDA stream passed in tp_run.stream (the
  *    caller's current stream).  Host-output calls synchronise that stream.
+ *    Resets, writes and reads on the device run on the legacy default stream;
+ *    runs of one scene, on whatever streams, wait for one another and for
+ *    these, and these for the runs before them.
  *  - Units: cm, Angstrom, 1/cm, barn, Angstrom^3, radians.
  *  - The library allocates its own device memory (cudaMalloc) for a scene.
  */

@@ -168,6 +168,9 @@ struct tp_scene {
   int* d_abort = nullptr;
   int test_flags = 0;   // tp_set_test_flags
   cudaEvent_t stage_done = nullptr;
+  // runs on a stream that the legacy default stream does not wait for
+  cudaEvent_t default_done = nullptr, side_done = nullptr;
+  bool default_work = true, side_work = false;   // work of this scene since the event was recorded / joined
   bool stage_pending = false;
   // launch configuration: last used, and the autotuned choice per gradient mode
   int kernel = 0, block = 0, ctas_per_sm = 0;
@@ -191,6 +194,57 @@ struct tp_scene {
 };
 
 namespace {
+
+// A scene's work lies on the caller's streams (runs) and on the legacy default
+// stream (resets, writes, reads).  A run on another stream waits for the work
+// before it, wherever that is; side_ran then notes the run, and what
+// follows elsewhere waits for it (wait_side).  Default-stream runs need and pay
+// nothing.  A stream that the caller is capturing is left as it is.
+bool on_default(cudaStream_t st) { return st == nullptr || st == cudaStreamLegacy; }
+
+tp_status stream_captured(cudaStream_t st, bool* yes) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  TP_CUDA(cudaStreamIsCapturing(st, &cs));
+  *yes = cs != cudaStreamCaptureStatusNone;
+  return TP_OK;
+}
+
+tp_status wait_side(tp_scene* s, cudaStream_t st) {
+  if (!s->side_work) return TP_OK;
+  TP_CUDA(cudaStreamWaitEvent(on_default(st) ? cudaStreamLegacy : st, s->side_done, 0));
+  if (on_default(st)) { s->side_work = false; s->default_work = true; }
+  return TP_OK;
+}
+
+tp_status run_begins(tp_scene* s, cudaStream_t st) {
+  if (on_default(st)) {
+    s->default_work = true;
+    return wait_side(s, st);
+  }
+  bool captured = false;
+  tp_status e = stream_captured(st, &captured);
+  if (e != TP_OK || captured) return e;
+  if (!s->default_done) {
+    TP_CUDA(cudaEventCreateWithFlags(&s->default_done, cudaEventDisableTiming));
+    TP_CUDA(cudaEventCreateWithFlags(&s->side_done, cudaEventDisableTiming));
+  }
+  if (s->default_work) {
+    TP_CUDA(cudaEventRecord(s->default_done, cudaStreamLegacy));
+    s->default_work = false;
+  }
+  TP_CUDA(cudaStreamWaitEvent(st, s->default_done, 0));
+  return wait_side(s, st);
+}
+
+tp_status side_ran(tp_scene* s, cudaStream_t st) {
+  if (on_default(st)) return TP_OK;
+  bool captured = false;
+  tp_status e = stream_captured(st, &captured);
+  if (e != TP_OK || captured) return e;
+  TP_CUDA(cudaEventRecord(s->side_done, st));
+  s->side_work = true;
+  return TP_OK;
+}
 
 // Words of a run's description: the work counter (0), prefix sums, first ids.
 size_t work_words(const tp_scene* s) { return 2 + 2 * (size_t)s->n_inst; }
@@ -739,6 +793,7 @@ tp_status upload_blob(tp_scene* s) {
     s->blob_cap = blob.size();
   }
   TP_CUDA(cudaMemcpy(s->d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice));
+  s->default_work = true;
   s->blob_bytes = (uint32_t)blob.size();
   s->blob_dirty = false;
   return TP_OK;
@@ -1397,6 +1452,7 @@ tp_status tp_set_params(tp_scene* s, const double* inst_params) {
   TP_CUDA(cudaDeviceSynchronize());
   const std::vector<uint8_t> pb = params_bytes(s->inst_params, s->precision);
   TP_CUDA(cudaMemcpy(s->d_params, pb.data(), pb.size(), cudaMemcpyHostToDevice));
+  s->default_work = true;
   if (moving) s->blob_dirty = true;   // bounding radii and neighbour lists depend on the radii
   return TP_OK;
 }
@@ -1407,6 +1463,7 @@ tp_status tp_reset_tallies(tp_scene* s) {
   TP_CUDA(cudaDeviceSynchronize());
   if (s->h_abort) *s->h_abort = 0;
   TP_CUDA(cudaMemset(s->d_sum, 0, s->clear_bytes));   // tallies, counters and status are one block
+  s->default_work = true;
   std::fill(s->n_done.begin(), s->n_done.end(), 0.0);
   return TP_OK;
 }
@@ -1444,6 +1501,8 @@ tp_status tp_run_histories(tp_scene* s, const tp_run* r) {
   if (r->stage < 0 || r->stage > 2) return fail(TP_ERR_INVALID_ARG, "stage %d: need 0, 1 or 2", r->stage);
   if (r->stage != 0 && r->kernel == TP_KERNEL_AUTO)
     return fail(TP_ERR_INVALID_ARG, "stage %d needs an explicit kernel (the autotuner picks the staging)", r->stage);
+  tp_status ordered = run_begins(s, st);
+  if (ordered != TP_OK) return ordered;
   const bool tune = r->kernel == TP_KERNEL_AUTO && s->tuned_kernel[grad] == 0;
   if (grad && (r->secondaries == 2 || (r->secondaries == 0 && (tune || (r->kernel == TP_KERNEL_AUTO && s->tuned_defer))))) {
     tp_status e = ensure_sec(s, total);   // before any capture: it may allocate
@@ -1485,6 +1544,8 @@ tp_status tp_run_histories(tp_scene* s, const tp_run* r) {
     cudaError_t ce = launch_cfg(s, cfg, grad, r->seed, total, r->records, r->n_records, o, st, true);
     if (ce != cudaSuccess) return fail(TP_ERR_CUDA, "transport launch: %s", cudaGetErrorString(ce));
   }
+  e = side_ran(s, st);
+  if (e != TP_OK) return e;
   for (int i = 0; i < s->n_inst; ++i) s->n_done[i] += (double)r->n_histories[i];
   s->kernel = cfg.kernel;
   s->block = cfg.block;
@@ -1507,6 +1568,9 @@ tp_status tp_read_tallies(tp_scene* s, int tally, int instance, double* mean, do
   const int nb = s->tallies[tally].nbins[0] * s->tallies[tally].nbins[1];
   const size_t off = (size_t)instance * s->total_bins + s->tally_off[tally];
   const double n = s->n_done[instance];
+  tp_status ordered = wait_side(s, nullptr);
+  if (ordered != TP_OK) return ordered;
+  s->default_work = true;
   if (on_device) {
     TP_CUDA(launch_stats(s->d_sum + off, s->d_sumsq + off, n, nb, mean, err, 0));
     return TP_OK;
@@ -1558,6 +1622,7 @@ tp_status tp_write_raw(tp_scene* s, int instance, const double* sum, const doubl
     if (J) TP_CUDA(cudaMemcpy(s->d_J + dst, J + p * nb, nb * sizeof(double), kind));
     if (J2) TP_CUDA(cudaMemcpy(s->d_J2 + dst, J2 + p * nb, nb * sizeof(double), kind));
   }
+  s->default_work = true;
   s->n_done[instance] = n_histories;
   return TP_OK;
 }
@@ -1570,6 +1635,8 @@ tp_status tp_backward(tp_scene* s, const double* grad_tallies, double* grad_para
   const int ni = s->n_inst, np = s->n_par;
   // d/dtheta: radius per cm; scale and density are log-parameters in the
   // accumulators, divided by the parameter value here
+  tp_status ordered = run_begins(s, st);
+  if (ordered != TP_OK) return ordered;
   TP_CUDA(cudaStreamSynchronize(st));
   for (int i = 0; i < ni; ++i) {
     for (int p = 0; p < np; ++p) {
@@ -1673,6 +1740,8 @@ void tp_destroy_scene(tp_scene* s) {
   if (s->h_aux) cudaFreeHost(s->h_aux);
   if (s->h_abort) cudaFreeHost(const_cast<int*>(s->h_abort));
   if (s->stage_done) cudaEventDestroy(s->stage_done);
+  if (s->default_done) cudaEventDestroy(s->default_done);
+  if (s->side_done) cudaEventDestroy(s->side_done);
   delete s;
 }
 

@@ -258,10 +258,15 @@ class Scene:
     def means(self) -> torch.Tensor:
         """Per-instance means of every bin, [n_inst, total_bins] float64 on the GPU."""
         out = torch.empty(self.n_inst, self.total_bins, dtype=torch.float64, device="cuda")
+        side = _stream_handle(None) != 0   # the reads run on the default stream
+        if side:
+            torch.cuda.current_stream().synchronize()
         for q in range(self.n_inst):
             for t in range(len(self.tally_bins)):
                 o = self.tally_off[t]
                 N.tp_read_tallies(self.handle, t, q, out[q, o:].data_ptr(), None, True)
+        if side:
+            torch.cuda.default_stream().synchronize()
         return out
 
     def backward(self, grad: torch.Tensor, stream=None) -> torch.Tensor:

@@ -97,3 +97,27 @@ def test_tables_change_behind_a_run_in_flight_on_a_side_stream(grid):
         seen.append((sc.raw(), sc.counters()))
     same(sc, seen[0])
     sc.close()
+
+
+def test_reset_runs_and_reads_on_several_streams_are_ordered():
+    """Reset, two runs on two side streams, one on the default stream, the means and
+    the backward pass, with no wait by the caller: what a single stream gives."""
+    from paper_2304_06226_gb300.engine import Scene
+    d = W.imaging(n_prims=30, precision="f64", psd_bins=64)
+    sc, seen = Scene(d), []
+    for streams in ((None,) * 3, (torch.cuda.Stream(), torch.cuda.Stream(), None)):
+        sc.run(1000, kernel=1, want_grad=True)
+        sc.reset()
+        for k, (st, n) in enumerate(zip(streams, (300_000, 200_000, 100_000))):
+            sc.run(n, first=10**6 * k, kernel=1, want_grad=True, stream=st)
+        means = sc.means()
+        with torch.cuda.stream(streams[0] or torch.cuda.default_stream()):
+            grad = sc.backward(torch.ones_like(means))
+        torch.cuda.synchronize()
+        seen.append((means.cpu().numpy(), grad.cpu().numpy(), sc.counters()))
+    sc.close()
+    (m0, g0, c0), (m1, g1, c1) = seen
+    assert c0 == c1 and c0["histories"] == 600_000
+    assert m0.any() and np.allclose(m1, m0, rtol=1e-11, atol=1e-11 * m0.max())
+    # a gradient's terms cancel: rounding against the sum of their magnitudes, below 100 a history
+    assert np.allclose(g1, g0, rtol=0.0, atol=1e-9)
