@@ -78,7 +78,7 @@ template <> struct Tr<float> {
   }
   // 1/x, sqrt(x) and 1/sqrt(x) of the special-function unit, without the
   // scaling of subnormal operands that division and square root carry under
-  // this unit's flags (2 ulp): on normal operands quot(a, rcp(b)), root(x) and
+  // this unit's flags (2 ulp): on normal operands quot(a, divisor(b)), root(x) and
   // rroot(x) are bit for bit what a / b, sqrtf(x) and 1 / sqrtf(x) give
   // (compared on 6.7e7 operands over 2^-60 .. 2^60), in two instructions
   // instead of eight.  For lengths, directions and cross sections, which are
@@ -103,7 +103,9 @@ template <> struct Tr<float> {
   // Sums of products below name the product that is rounded by itself, so that
   // a neutron's path does not depend on what the compiler contracts where:
   // every kernel and build gives the same path bit for bit.
-  static __device__ __forceinline__ float quot(float a, float inv) { return __fmul_rn(a, inv); }
+  // a / b, where several quotients may share divisor(b): here its reciprocal
+  static __device__ __forceinline__ float divisor(float b) { return rcp(b); }
+  static __device__ __forceinline__ float quot(float a, float d) { return __fmul_rn(a, d); }
   static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
   static __device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
   static constexpr float kPi = 3.14159265358979323846f;
@@ -122,7 +124,9 @@ template <> struct Tr<double> {
   static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
   static __device__ __forceinline__ double root(double x) { return sqrt(x); }
   static __device__ __forceinline__ double rroot(double x) { return 1.0 / sqrt(x); }
-  static __device__ __forceinline__ double quot(double a, double inv) { return a * inv; }
+  // (a reciprocal times a is rounded twice: quotients are divisions)
+  static __device__ __forceinline__ double divisor(double b) { return b; }
+  static __device__ __forceinline__ double quot(double a, double d) { return a / d; }
   static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
   static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
   static constexpr double kPi = 3.14159265358979323846;
@@ -395,13 +399,13 @@ __device__ __forceinline__ bool hit_terms(const Quad<R>& Q, R r, R* qq, R* C) {
   return true;
 }
 
-// Both intersections, nearer first; inv_A = 1 / A, shared by the radii of a shell.
+// Both intersections, nearer first; div_A = divisor(A), shared by the radii of a shell.
 template <bool FUSED, typename R>
-__device__ __forceinline__ bool hit_radius(const Quad<R>& Q, R inv_A, R r, R* t0, R* t1) {
+__device__ __forceinline__ bool hit_radius(const Quad<R>& Q, R div_A, R r, R* t0, R* t1) {
   R qq, C;
   if (!hit_terms<FUSED>(Q, r, &qq, &C)) return false;
   const bool some = qq != R(0);
-  const R a = some ? Tr<R>::quot(qq, inv_A) : R(0), b = some ? Tr<R>::quot(C, Tr<R>::rcp(qq)) : R(0);
+  const R a = some ? Tr<R>::quot(qq, div_A) : R(0), b = some ? Tr<R>::quot(C, Tr<R>::divisor(qq)) : R(0);
   *t0 = fmin(a, b);
   *t1 = fmax(a, b);
   return true;
@@ -420,7 +424,7 @@ __device__ __forceinline__ bool hit_far(const Quad<R>& Q, R r, R* t1) {
     const bool neg = signbit(Q.B);
     t = (neg ? qq : C) / (neg ? Q.A : qq);
   } else {
-    t = fmax(Tr<R>::quot(qq, Tr<R>::rcp(Q.A)), Tr<R>::quot(C, Tr<R>::rcp(qq)));
+    t = fmax(Tr<R>::quot(qq, Tr<R>::divisor(Q.A)), Tr<R>::quot(C, Tr<R>::divisor(qq)));
   }
   *t1 = qq != R(0) ? t : R(0);
   return true;
@@ -432,8 +436,8 @@ template <typename R>
 __device__ __forceinline__ bool hit_near(const Quad<R>& Q, R r, R* t0) {
   R qq, C;
   if (!(Q.B < R(0)) || !hit_terms<true>(Q, r, &qq, &C) || !(C >= R(0))) return false;
-  const R t = Tr<R>::quot(C, Tr<R>::rcp(qq));
-  *t0 = sizeof(R) == 8 ? t : fmin(Tr<R>::quot(qq, Tr<R>::rcp(Q.A)), t);
+  const R t = Tr<R>::quot(C, Tr<R>::divisor(qq));
+  *t0 = sizeof(R) == 8 ? t : fmin(Tr<R>::quot(qq, Tr<R>::divisor(Q.A)), t);
   return true;
 }
 
@@ -475,7 +479,7 @@ __device__ R exit_dist(const DPrim<R>& p, R dR, const R x[3], const R u[3], int*
     } else {
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const R t = Tr<R>::quot(copysign(p.p[a], v[a]) - q[a], Tr<R>::rcp(v[a]));
+        const R t = Tr<R>::quot(copysign(p.p[a], v[a]) - q[a], Tr<R>::divisor(v[a]));
         if (v[a] != R(0) && t < best) { best = t; bf = 2 * a + (v[a] > R(0) ? 1 : 0); }
       }
     }
@@ -487,7 +491,7 @@ __device__ R exit_dist(const DPrim<R>& p, R dR, const R x[3], const R u[3], int*
     if (hit_far(Q, rr.r1, &t) && t >= R(0) && t < best) { best = t; bf = 0; }
     if (rr.r0 > R(0) && hit_near(Q, rr.r0, &t) && t < best) { best = t; bf = 1; }
     if (tube && v[2] != R(0)) {
-      t = Tr<R>::quot(copysign(rr.h, v[2]) - q[2], Tr<R>::rcp(v[2]));
+      t = Tr<R>::quot(copysign(rr.h, v[2]) - q[2], Tr<R>::divisor(v[2]));
       if (t < best) { best = t; bf = v[2] > R(0) ? 3 : 2; }
     }
   }
@@ -515,7 +519,7 @@ __device__ R entry_dist(const DPrim<R>& p, R dR, const R x[3], const R u[3], int
         continue;
       }
       const R inv = Tr<R>::rcp(v[a]);
-      R ta = Tr<R>::quot(-p.p[a] - q[a], inv), tb = Tr<R>::quot(p.p[a] - q[a], inv);
+      R ta = Tr<R>::mul(-p.p[a] - q[a], inv), tb = Tr<R>::mul(p.p[a] - q[a], inv);
       int fa = 2 * a;
       if (ta > tb) { const R t = ta; ta = tb; tb = t; fa = 2 * a + 1; }
       if (ta > tn) { tn = ta; fn = fa; }
@@ -528,12 +532,12 @@ __device__ R entry_dist(const DPrim<R>& p, R dR, const R x[3], const R u[3], int
   const bool tube = p.shape == TP_TUBE;
   const Radii<R> rr = radii(p, dR);
   const Quad<R> Q = quad(q, v, tube);
-  const R inv_A = Tr<R>::rcp(Q.A);
+  const R div_A = Tr<R>::divisor(Q.A);
   R o0, o1;
   if (Q.A == R(0)) {
     if (Q.C2 > rr.r1 * rr.r1) return INF;
     o0 = -INF; o1 = INF;
-  } else if (!hit_radius<false>(Q, inv_A, rr.r1, &o0, &o1)) {
+  } else if (!hit_radius<false>(Q, div_A, rr.r1, &o0, &o1)) {
     return INF;
   }
   R z0 = -INF, z1 = INF;
@@ -542,8 +546,8 @@ __device__ R entry_dist(const DPrim<R>& p, R dR, const R x[3], const R u[3], int
     if (v[2] == R(0)) {
       if (fabs(q[2]) > rr.h) return INF;
     } else {
-      const R inv = Tr<R>::rcp(v[2]);
-      const R ta = Tr<R>::quot(-rr.h - q[2], inv), tb = Tr<R>::quot(rr.h - q[2], inv);
+      const R dv = Tr<R>::divisor(v[2]);
+      const R ta = Tr<R>::quot(-rr.h - q[2], dv), tb = Tr<R>::quot(rr.h - q[2], dv);
       if (ta < tb) { z0 = ta; z1 = tb; fz0 = 2; } else { z0 = tb; z1 = ta; fz0 = 3; }
     }
   }
@@ -551,7 +555,7 @@ __device__ R entry_dist(const DPrim<R>& p, R dR, const R x[3], const R u[3], int
   int f0 = 0, f1 = 1;
   if (rr.r0 > R(0)) {
     R i0, i1;
-    if (Q.A > R(0) && hit_radius<true>(Q, inv_A, rr.r0, &i0, &i1)) {
+    if (Q.A > R(0) && hit_radius<true>(Q, div_A, rr.r0, &i0, &i1)) {
       e0 = i0; s1 = i1; e1 = o1;
     } else if (Q.A == R(0) && Q.C2 < rr.r0 * rr.r0) {
       return INF;
@@ -801,7 +805,7 @@ __device__ __forceinline__ int tally_bin(const DTally<R>& T, R x0, R x1, R x2, R
         // elastic momentum transfer Q = 4 pi sin(theta/2) / lambda (Eq. eQelastic)
         R sh, ch;
         d_sincos(R(0.5) * tally_angle(T, x0, x1, x2), &sh, &ch);
-        return bin1(Tr<R>::quot(Tr<R>::kFourPi * sh, Tr<R>::rcp(lam)), T.lo[0], T.hi[0], T.inv_w[0], T.nb0);
+        return bin1(Tr<R>::quot(Tr<R>::kFourPi * sh, Tr<R>::divisor(lam)), T.lo[0], T.hi[0], T.inv_w[0], T.nb0);
       }
       case TP_TALLY_PSD: {
         const int bx = bin1(x0, T.lo[0], T.hi[0], T.inv_w[0], T.nb0);
@@ -903,7 +907,7 @@ __device__ bool source(const KParams<R>& kp, const View<R>& V, Particle<R>& P, R
       R sc, cc;
       d_sincos(R(0.5) * Tr<R>::kPi * Tr<R>::u01(b.w), &sc, &cc);
       const R e = kp.src_kT * (-d_log(Tr<R>::u01(a.z)) - d_log(Tr<R>::u01(a.w)) * cc * cc);
-      P.lam = Tr<R>::root(Tr<R>::quot(R(kH2over2mn), Tr<R>::rcp(e)));
+      P.lam = Tr<R>::root(Tr<R>::quot(R(kH2over2mn), Tr<R>::divisor(e)));
     } else {
       P.lam = kp.src_lam_hi > kp.src_lam_lo ? kp.src_lam_lo + (kp.src_lam_hi - kp.src_lam_lo) * Tr<R>::u01(a.z)
                                             : kp.src_lam_lo;
@@ -980,7 +984,7 @@ __device__ __forceinline__ void scatter_dir(const View<R>& V, int mat, int proc,
       const int mid = (lo + hi) >> 1;
       if (target < cum[mid + 1]) hi = mid; else lo = mid + 1;
     }
-    const R sb = Tr<R>::quot(lam, Tr<R>::rcp(R(2) * V.line_d[m.line_off + lo]));
+    const R sb = Tr<R>::quot(lam, Tr<R>::divisor(R(2) * V.line_d[m.line_off + lo]));
     rotate(u, Tr<R>::fma(R(-2) * sb, sb, R(1)), xphi);
   }
 }
@@ -1003,8 +1007,8 @@ __device__ __forceinline__ bool radius_crossing(const KParams<R>& kp, const View
   R si[TP_NPROC] = {R(0), R(0), R(0)}, so[TP_NPROC] = {R(0), R(0), R(0)};
   if (mi >= 0) sigma(V, mi, ip, P.lam, si);
   if (mo >= 0) sigma(V, mo, ip, P.lam, so);
-  const R inv_cosn = Tr<R>::rcp(cosn);
-  add_at(P.A, kp.radius_par, Tr<R>::quot(-((si[0] + si[1] + si[2]) - (so[0] + so[1] + so[2])), inv_cosn));
+  const R div_cosn = Tr<R>::divisor(cosn);
+  add_at(P.A, kp.radius_par, Tr<R>::quot(-((si[0] + si[1] + si[2]) - (so[0] + so[1] + so[2])), div_cosn));
   const R term[4] = {si[TP_PROC_INC], si[TP_PROC_BRAGG], -so[TP_PROC_INC], -so[TP_PROC_BRAGG]};
   const R C = fabs(term[0]) + fabs(term[1]) + fabs(term[2]) + fabs(term[3]);
   if (!(C > R(0))) return false;
@@ -1026,7 +1030,7 @@ __device__ __forceinline__ bool radius_crossing(const KParams<R>& kp, const View
   const int mat = pick < 2 ? mi : mo;
   const int proc = (pick & 1) ? TP_PROC_BRAGG : TP_PROC_INC;
   *S = P;
-  S->w = Tr<R>::quot(P.w * (tp > R(0) ? R(1) : R(-1)) * C, inv_cosn);
+  S->w = Tr<R>::quot(P.w * (tp > R(0) ? R(1) : R(-1)) * C, div_cosn);
   S->nscat = P.nscat + 1;
   S->sub0 = 4u + 2u * P.nsec;
   S->k = 0;
@@ -1119,11 +1123,11 @@ __device__ __forceinline__ void grid_search(const KParams<R>& kp, const View<R>&
   R db = *db_io;
   int target = *target_io, face = *face_io;
   R t0 = R(0), t1 = db;
-  R inv_u[3];
+  R div_u[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const R inv = Tr<R>::rcp(u[a]);
-    inv_u[a] = inv;
+    if constexpr (sizeof(R) == 4) div_u[a] = inv; else div_u[a] = Tr<R>::divisor(u[a]);
     if (u[a] != R(0)) {
       R ta = (kp.grid_lo[a] - x[a]) * inv, tb = (kp.grid_hi[a] - x[a]) * inv;
       if (ta > tb) { const R t = ta; ta = tb; tb = t; }
@@ -1150,8 +1154,8 @@ __device__ __forceinline__ void grid_search(const KParams<R>& kp, const View<R>&
       const R next = Tr<R>::fma(R(up ? c + 1 : c), kp.grid_cell[a], kp.grid_lo[a]) - x[a];
       stp[a] = up ? stride : -stride;
       left[a] = up ? n - 1 - c : c;
-      tnext[a] = u[a] != R(0) ? Tr<R>::quot(next, inv_u[a]) : Tr<R>::inf();
-      tdel[a] = u[a] != R(0) ? fabs(Tr<R>::quot(kp.grid_cell[a], inv_u[a])) : Tr<R>::inf();
+      tnext[a] = u[a] != R(0) ? Tr<R>::quot(next, div_u[a]) : Tr<R>::inf();
+      tdel[a] = u[a] != R(0) ? fabs(Tr<R>::quot(kp.grid_cell[a], div_u[a])) : Tr<R>::inf();
     }
     int k = kp.grid_start[cell], k1 = kp.grid_start[cell + 1];
     bool fresh = true;      // the cell's list is not looked at yet
@@ -1251,7 +1255,7 @@ __device__ int advance(const KParams<R>& kp, const View<R>& V, Particle<R>& P, c
   R l = INF;
   if (sig_g > R(0)) {
     a.r0 = philox(make_uint4(P.k, P.sub0, P.hid, P.inst), kp.key0, kp.key1);
-    l = Tr<R>::quot(Tr<R>::neg_log_u01(a.r0.x), Tr<R>::rcp(sig_g));
+    l = Tr<R>::quot(Tr<R>::neg_log_u01(a.r0.x), Tr<R>::divisor(sig_g));
   }
   // next boundary
   R db;
@@ -1315,7 +1319,7 @@ __device__ __forceinline__ int reflect(const View<R>& V, Particle<R>& P, unsigne
   R n[3];
   normal(pt, P.x, face, n);
   const R un = dot3(P.u[0], n[0], P.u[1], n[1], P.u[2], n[2]);
-  const R Q = Tr<R>::quot(Tr<R>::kFourPi * fabs(un), Tr<R>::rcp(P.lam));
+  const R Q = Tr<R>::quot(Tr<R>::kFourPi * fabs(un), Tr<R>::divisor(P.lam));
   const R Rf = mirror_R(V.mirrors[pt.mirror], Q);
   cnt[C_MIRROR]++;
   P.w *= Rf;
