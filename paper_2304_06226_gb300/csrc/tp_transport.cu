@@ -756,8 +756,10 @@ __device__ __forceinline__ int bin1(R x, R lo, R hi, R inv_w, int n) {
 }
 
 // Bin of the angle between (x - origin) and the tally axis.  FP64: an FP32 angle
-// (good to 2e-6 rad) settles the bin unless it lies that near a bin's edge; then,
-// and only then, the FP64 angle is taken, so the bin is always the FP64 one.
+// (good to 2e-6 rad) settles the bin unless it lies that near a bin's edge or the
+// distance's square leaves the middle of the FP32 range (1e-10 to 1e15 cm; what
+// underflows in the cross product is then below 1e-9 rad); then, and only then,
+// the FP64 angle is taken, so the bin is always the FP64 one.
 template <typename R>
 __device__ __forceinline__ R tally_angle(const DTally<R>& T, R x0, R x1, R x2);
 
@@ -771,7 +773,9 @@ __device__ __forceinline__ int angle_bin(const DTally<R>& T, R x0, R x1, R x2) {
     const float w = (float)T.inv_w[0];
     const float y = (th - (float)T.lo[0]) * w, slack = 4e-6f * w + 1e-6f * (float)T.nb0;
     const float b = floorf(y);
-    if (y - b > slack && b + 1.0f - y > slack && b >= 0.0f && b < (float)T.nb0) return (int)b;
+    const float vv = v0 * v0 + v1 * v1 + v2 * v2;
+    if (y - b > slack && b + 1.0f - y > slack && b >= 0.0f && b < (float)T.nb0 && vv > 1e-20f && vv < 1e30f)
+      return (int)b;
   }
   return bin1(tally_angle(T, x0, x1, x2), T.lo[0], T.hi[0], T.inv_w[0], T.nb0);
 }
