@@ -37,6 +37,7 @@
 #include <type_traits>
 
 #include "tp_internal.h"
+#include "tp_box_exit.h"
 
 namespace tp {
 namespace {
@@ -466,16 +467,7 @@ __device__ R exit_dist(const DPrim<R>& p, R dR, const R x[3], const R u[3], int*
   int bf = -1;
   if (p.shape == TP_BOX) {
     if constexpr (sizeof(R) == 8) {
-      // the nearest of the three faces by cross-multiplication, one division
-      // (three reciprocals were a third of the FP64 instructions of a slab's flight)
-      R bn = R(1), bd = R(0);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const bool neg = signbit(v[a]);
-        const R n = p.p[a] + (neg ? q[a] : -q[a]), d = fabs(v[a]);
-        if (n * bd < bn * d) { bn = n; bd = d; bf = 2 * a + (neg ? 0 : 1); }
-      }
-      best = bf >= 0 ? bn / bd : best;
+      best = box_exit(p.p, q, v, best, &bf);
     } else {
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
