@@ -378,8 +378,16 @@ tp_status tp_abort(tp_scene* s);
  * TP_TEST_FULL_BUILD: the scene runs the kernels' complete feature build even
  * if the lean one serves it (the two must agree; the test of that uses it).
  * TP_TEST_SMALL_SEC_QUEUE: the queue of radius-derivative secondaries holds at
- * most 2^20 records, so that a short run goes through several chunks. */
-enum { TP_TEST_SKIP_TABLE_COPY = 1, TP_TEST_FULL_BUILD = 2, TP_TEST_SMALL_SEC_QUEUE = 4 };
+ * most 2^20 records, so that a short run goes through several chunks.
+ * TP_TEST_SMALL_HIST_INTERVAL: warp pools that count in shared memory empty
+ * their histogram into the tallies every 64 crossings of a warp instead of
+ * 2^23, which few runs reach before their end. */
+enum {
+  TP_TEST_SKIP_TABLE_COPY = 1,
+  TP_TEST_FULL_BUILD = 2,
+  TP_TEST_SMALL_SEC_QUEUE = 4,
+  TP_TEST_SMALL_HIST_INTERVAL = 8
+};
 tp_status tp_set_test_flags(tp_scene* s, int flags);
 
 /* Launch configuration of the last run: kernel (TP_KERNEL_*), block size and
@@ -390,6 +398,12 @@ tp_status tp_get_launch(tp_scene* s, int* kernel, int* block_size, int* ctas_per
  * secondaries two per chunk of histories (first pass, second pass); 0 before
  * any run or if the run had no histories.  No device work. */
 int tp_get_launch_count(const tp_scene* s);
+
+/* 1 if the last tp_run_histories counted its scores in shared memory instead of
+ * summing weights: warp pools, no gradients, one instance, at most 4096 bins,
+ * every weight 1 (no biased process, no mirror), no grid.  The tallies are the
+ * same whole numbers.  0 otherwise.  No device work. */
+int tp_get_launch_counting(const tp_scene* s);
 
 /* The complete launch configuration of the scene's last tp_run_histories
  * (after the autotuner, if it ran): transport kernel (TP_KERNEL_*), threads

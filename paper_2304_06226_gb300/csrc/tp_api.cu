@@ -888,14 +888,24 @@ tp_status pick_launch(tp_scene* s, bool grad, int req_block, int req_ctas, int* 
   return TP_OK;
 }
 
-// Bins of a histogram in shared memory: 16 KB a block leave the warp pools
-// their four blocks of 256 threads per SM (54 of 57 KB a block).
+// Bins of a histogram in shared memory: 16 KB a block leave FP32 warp pools
+// with tables of up to 3 KB their four blocks of 256 threads per SM (54 of 57 KB
+// a block); FP64 pools (55 KB without it) and larger tables keep three.
 constexpr int kCountBinsMax = 4096;
+
+// A crossing scores at most twice in one bin.  A warp empties its block's histogram
+// at the first refill after kHistInterval of its crossings; until the next refill,
+// or the run's end, the 64 neutrons of its pool make at most 64 x event_cap more.
+// Eight warps then add less than 8 x 2 x (2^23 + 64 x 2^21) < 2^32 to a count.
+constexpr unsigned kHistInterval = 1u << 23, kHistIntervalTest = 64;
+constexpr int kCountEventCapMax = 1 << 21;
 
 // True if plain runs of the warp pools may count instead of summing weights: no
 // process is biased and no surface reflects, so every weight stays exactly 1.
 bool counts_only(const tp_scene* s) {
-  if (s->n_inst != 1 || s->total_bins < 1 || s->total_bins > kCountBinsMax || s->grid_cells > 0) return false;
+  if (s->n_inst != 1 || s->total_bins < 1 || s->total_bins > kCountBinsMax || s->grid_cells > 0 ||
+      s->event_cap > kCountEventCapMax)
+    return false;
   for (const tp_prim& p : s->prims)
     if (p.mirror >= 0) return false;
   for (const Mat& m : s->mats)
@@ -994,6 +1004,7 @@ cudaError_t launch_one(tp_scene* s, const LaunchCfg& c, bool grad, uint64_t seed
   k.regroup = c.regroup;
   const int grid = s->sm_count * c.ctas;
   const long long warps = (long long)grid * (c.block / 32);
+  k.hist_interval = (s->test_flags & TP_TEST_SMALL_HIST_INTERVAL) ? kHistIntervalTest : kHistInterval;
   k.chunk = sec_mode == 2 ? 16 : (int)std::max(1ll, std::min(256ll, (long long)(total / (unsigned long long)(warps * 8))));
   // the first launch after the run's description finds the counter at 0
   cudaError_t e = first ? cudaSuccess : cudaMemsetAsync(s->d_work, 0, sizeof(unsigned long long), st);
@@ -1685,7 +1696,7 @@ tp_status tp_abort(tp_scene* s) {
 
 tp_status tp_set_test_flags(tp_scene* s, int flags) {
   g_err.clear();
-  if (flags & ~(TP_TEST_SKIP_TABLE_COPY | TP_TEST_FULL_BUILD | TP_TEST_SMALL_SEC_QUEUE))
+  if (flags & ~(TP_TEST_SKIP_TABLE_COPY | TP_TEST_FULL_BUILD | TP_TEST_SMALL_SEC_QUEUE | TP_TEST_SMALL_HIST_INTERVAL))
     return fail(TP_ERR_INVALID_ARG, "unknown test flags %#x", flags);
   if (!s) {
     g_noalloc_test_flags.store(flags & TP_TEST_SKIP_TABLE_COPY);
@@ -1699,6 +1710,8 @@ tp_status tp_set_test_flags(tp_scene* s, int flags) {
 }
 
 int tp_get_launch_count(const tp_scene* s) { return s ? s->launches : 0; }
+
+int tp_get_launch_counting(const tp_scene* s) { return s ? s->last_cfg.count : 0; }
 
 tp_status tp_get_launch_info(const tp_scene* s, tp_launch_info* out) {
   if (!s || !out) return fail(TP_ERR_INVALID_ARG, "null argument");

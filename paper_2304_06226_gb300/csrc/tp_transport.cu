@@ -2181,12 +2181,6 @@ __device__ __forceinline__ int pool_collide(const KParams<R>& kp, const View<R>&
   return Q_ADVP;
 }
 
-// A lane scores at most twice in a bin per crossing, so between two emptyings
-// of the block's histogram (each warp empties it once a lane of it has made
-// another 2^kHistShift crossings, at its next refill, at most a pool's events
-// later) a count stays below 2^30.
-constexpr int kHistShift = 18;
-
 // Adds the block's counts to the tallies and clears them: threads i0, i0 + step, ..
 template <typename R>
 __device__ __forceinline__ void empty_hist(const KParams<R>& kp, unsigned* hist, int i0, int step) {
@@ -2248,7 +2242,7 @@ __global__ void __launch_bounds__(256, MINB) k_transport_wq(const __grid_constan
   for (int i = 0; i < kPool; i += 32) stack[Q_EMPTY * kPool + i + lane] = (uint8_t)(i + lane);
   unsigned counts = (unsigned)kPool << (8 * Q_EMPTY);   // warp-uniform
   bool work_left = true;                                // warp-uniform
-  unsigned emptied = 0;                                 // kOptCount: crossings >> kHistShift at the last emptying
+  unsigned emptied = 0;                                 // kOptCount: the warp's crossings at its last emptying
 
   for (;;) {
     __syncwarp();   // the last step's pushes and stores
@@ -2285,10 +2279,10 @@ __global__ void __launch_bounds__(256, MINB) k_transport_wq(const __grid_constan
       }
       work_left = __all_sync(kFull, slot < 0 || g < total) != 0;
       if constexpr ((OPT & kOptCount) != 0) {
-        // long before a 32-bit count could run over (no run of ordinary size
-        // gets there), the histogram is emptied into the tallies
-        const unsigned now = __reduce_max_sync(kFull, cnt[C_CROSS] >> kHistShift);
-        if (now != emptied) {
+        // long before a 32-bit count could run over (kHistInterval), the
+        // histogram is emptied into the tallies
+        const unsigned now = __reduce_add_sync(kFull, cnt[C_CROSS]);
+        if (now - emptied >= kp.hist_interval) {
           emptied = now;
           empty_hist(kp, V.hist, lane, 32);
         }

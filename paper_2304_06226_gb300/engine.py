@@ -255,6 +255,10 @@ class Scene:
         """Transport kernels the last run launched (two per chunk with queued secondaries)."""
         return N.tp_get_launch_count(self.handle)
 
+    def launch_counting(self) -> bool:
+        """Whether the last run counted its scores in shared memory (tp_get_launch_counting)."""
+        return bool(N.tp_get_launch_counting(self.handle))
+
     def means(self) -> torch.Tensor:
         """Per-instance means of every bin, [n_inst, total_bins] float64 on the GPU."""
         out = torch.empty(self.n_inst, self.total_bins, dtype=torch.float64, device="cuda")

@@ -17,6 +17,7 @@ STATUS_NAMES = ["TP_OK", "TP_ERR_INVALID_ARG", "TP_ERR_GEOMETRY", "TP_ERR_CUDA",
 TP_TEST_SKIP_TABLE_COPY = 1
 TP_TEST_FULL_BUILD = 2
 TP_TEST_SMALL_SEC_QUEUE = 4
+TP_TEST_SMALL_HIST_INTERVAL = 8
 TP_BOX, TP_TUBE, TP_SPHERE = 0, 1, 2
 TP_ROLE_BULK, TP_ROLE_DETECTOR, TP_ROLE_BLACK = 0, 1, 2
 TP_PROC_ABS, TP_PROC_INC, TP_PROC_BRAGG, TP_NPROC = 0, 1, 2, 3
@@ -133,6 +134,7 @@ SIGNATURES = {
     "tp_get_launch": (C.c_int, [SCENE_P, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int)]),
     "tp_total_bins": (C.c_int, [SCENE_P]),
     "tp_get_launch_count": (C.c_int, [SCENE_P]),
+    "tp_get_launch_counting": (C.c_int, [SCENE_P]),
     "tp_get_launch_info": (C.c_int, [SCENE_P, C.POINTER(tp_launch_info)]),
     "tp_abort": (C.c_int, [SCENE_P]),
     "tp_measure_peaks": (C.c_int, [C.POINTER(tp_peaks), C.c_void_p]),
@@ -268,6 +270,10 @@ def tp_get_launch_info(scene: int) -> dict:
 
 def tp_get_launch_count(scene: int) -> int:
     return lib.tp_get_launch_count(scene)
+
+
+def tp_get_launch_counting(scene: int) -> int:
+    return lib.tp_get_launch_counting(scene)
 
 
 def tp_total_bins(scene: int) -> int:

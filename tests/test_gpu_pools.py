@@ -103,3 +103,67 @@ def test_counting_adds_to_what_is_there_and_stops_with_a_bias():
     raw = sc.raw()
     sc.close()
     assert not (raw["sum"] == raw["sumsq"]).all()
+
+
+def _counting(desc, n=1000, **kw):
+    from paper_2304_06226_gb300.engine import Scene
+    sc = Scene(desc)
+    sc.run(n, kernel=3, **kw)
+    torch.cuda.synchronize()
+    form = sc.launch_counting()
+    sc.close()
+    return form
+
+
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+def test_which_scenes_count(precision):
+    assert all(_counting(UNIT[k](precision)) for k in UNIT if k != "powder_4097")
+    assert not _counting(UNIT["powder_4097"](precision))
+    assert not _counting(W.guide(precision=precision))                      # mirrors
+    assert not _counting(W.slab(g=3.0, precision=precision))                # a bias
+    assert not _counting(W.imaging(n_prims=60, precision=precision, psd_bins=16))   # a grid
+    grad = W.imaging(n_prims=10, precision=precision, psd_bins=16)          # no grid, no bias
+    grad["bias"][:] = 1.0
+    assert _counting(grad) and not _counting(grad, want_grad=True)
+
+
+@pytest.mark.parametrize("cap,form", [(1 << 21, True), ((1 << 21) + 1, False), (2**31 - 1, False)])
+def test_counting_stops_above_the_event_cap_its_bound_is_for(cap, form):
+    """A count stays below 2^32 while no history has more events than this."""
+    desc = W.powder()
+    desc["event_cap"] = cap
+    assert _counting(desc) is form
+
+
+def test_a_bias_set_later_ends_counting_and_none_brings_it_back():
+    from paper_2304_06226_gb300.engine import Scene
+    sc, seen = Scene(W.powder()), []
+    for g in (1.0, 2.0, 1.0):
+        sc.set_bias(0, (1.0, g, 1.0))
+        sc.run(1000, kernel=3)
+        seen.append(sc.launch_counting())
+    sc.close()
+    assert seen == [True, False, True]
+
+
+@pytest.mark.parametrize("block", [32, 160, 256])
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+@pytest.mark.parametrize("scene", ["powder_4096", "orders", "chopper", "slab"])
+def test_histogram_emptied_while_the_block_scores(scene, precision, block):
+    """Every warp empties its block's histogram many times while the others score
+    (the flag's 64 crossings instead of 2^23): no count is lost or added twice."""
+    from paper_2304_06226_gb300 import native as N
+    from paper_2304_06226_gb300.engine import Scene
+    n = 1_000_001
+    desc = UNIT[scene](precision)
+    sc = Scene(desc)
+    sc.set_test_flags(N.TP_TEST_SMALL_HIST_INTERVAL)
+    sc.run(n, kernel=3, block_size=block, ctas_per_sm=1)
+    torch.cuda.synchronize()
+    assert sc.launch_counting()
+    got, cnt = sc.raw(), sc.counters()
+    assert cnt["crossings"] > 10 * 64 * 152 * (block // 32)   # ten times a warp and more
+    sc.close()
+    ref_cnt, ref = _run(desc, n, 2, 256)
+    assert cnt == ref_cnt
+    assert (got["sum"] == ref["sum"][0]).all() and (got["sumsq"] == ref["sumsq"][0]).all()
