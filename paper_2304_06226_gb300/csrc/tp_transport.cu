@@ -57,7 +57,12 @@ constexpr unsigned kFull = 0xffffffffu;
 // place and the secondary's state drop out of the registers.
 // kOptCount (plain runs of the warp pools in scenes whose weights stay 1): the
 // tallies are histograms of counts in shared memory, see score.
-constexpr int kOptGrid = 1, kOptFull = 2, kOptNoSec = 4, kOptCount = 8;
+// kOptUnroll (80-register FP32 build of the plain history kernel): the group
+// sum's loop is left to the compiler's unrolling.  There it pays (guide of 2e7
+// histories 6.22 -> 5.75 ms, with powder the same and total scattering 2.02 -> 2.08 ms);
+// the 64-register build and the other kernels are better off with the short
+// loop (powder 3.28 against 3.43 ms, guide 5.38 against 5.52 ms).
+constexpr int kOptGrid = 1, kOptFull = 2, kOptNoSec = 4, kOptCount = 8, kOptUnroll = 16;
 
 // ---------------------------------------------------------------------------
 // Precision traits
@@ -718,12 +723,11 @@ __device__ __forceinline__ AggGroup agg_group(unsigned long long idx) {
 // 2^k - 1 members, so the lowest member ends with the group's sum; the FP64
 // pipe is a small fraction of the FP32 one) and its lowest lane adds them
 // with one FP64 atomic per array.
-template <typename R>
+template <int OPT, typename R>
 __device__ __forceinline__ void agg_add2(const AggGroup& G, double* a, double* b, unsigned long long idx, R v,
                                          R v2) {
   int nx = G.next;
-#pragma unroll 1
-  for (int k = 0; k < G.rounds; ++k) {
+  auto jump = [&] {
     const int src = nx >= 0 ? nx : (int)(threadIdx.x & 31);
     const R x = __shfl_sync(G.am, v, src);
     const R y = __shfl_sync(G.am, v2, src);
@@ -733,6 +737,12 @@ __device__ __forceinline__ void agg_add2(const AggGroup& G, double* a, double* b
       v2 += y;
       nx = nn;
     }
+  };
+  if constexpr ((OPT & kOptUnroll) != 0) {
+    for (int k = 0; k < G.rounds; ++k) jump();
+  } else {
+#pragma unroll 1
+    for (int k = 0; k < G.rounds; ++k) jump();
   }
   if ((int)(threadIdx.x & 31) == __ffs(G.grp) - 1) {
     atomicAdd(a + idx, (double)v);
@@ -839,21 +849,22 @@ __device__ __forceinline__ void score_out(const KParams<R>& kp, const DTally<R>*
     // one grouping of the lanes on this path serves every array of the bin
     if (!secondary) {
       const AggGroup G = agg_group(idx);
-      agg_add2(G, kp.sum, kp.sumsq, idx, w, w * w);
+      agg_add2<OPT>(G, kp.sum, kp.sumsq, idx, w, w * w);
       if (GRAD) {
 #pragma unroll 1
         for (int p = 0; p < kp.npar; ++p) {
           const R g = w * sel(A, p, R(0));
-          agg_add2(G, kp.J, kp.J2, p * stride + idx, g, g * g);
+          agg_add2<OPT>(G, kp.J, kp.J2, p * stride + idx, g, g * g);
         }
       }
     } else if (kp.radius_par >= 0) {   // a radius-derivative secondary
       const AggGroup G = agg_group(idx);
-      agg_add2(G, kp.J, kp.J2, kp.radius_par * stride + idx, w, w * w);
+      agg_add2<OPT>(G, kp.J, kp.J2, kp.radius_par * stride + idx, w, w * w);
     }
   }
 }
 
+// The scores of one crossing: the tallies in `mask` whose filters it passes.
 //
 // With kOptCount every weight is 1 (no process is biased and nothing reflects),
 // so sum w and sum w^2 of a bin are both its count: a score is one shared-memory
@@ -1714,7 +1725,8 @@ __global__ void __launch_bounds__(256, MINB) k_transport(const __grid_constant__
     if (__all_sync(kFull, done)) break;
     if (alive) {
       bool spawn = false;
-      const int end = step<R, GRAD, OPT>(kp, V, P, ip, dR, cnt, &S, &spawn);
+      constexpr int kStepOpt = OPT | (MINB == 3 && sizeof(R) == 4 && !GRAD ? kOptUnroll : 0);
+      const int end = step<R, GRAD, kStepOpt>(kp, V, P, ip, dR, cnt, &S, &spawn);
       if (end >= 0) finish(kp, P, end);
       if (GRAD && spawn && sec_push(kp, S)) spawn = false;
       if (GRAD && spawn) {
