@@ -114,6 +114,10 @@ template <> struct Tr<float> {
   static __device__ __forceinline__ float quot(float a, float d) { return __fmul_rn(a, d); }
   static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
   static __device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+  // A ray whose squared transverse direction is no larger runs along the tube's
+  // axis: it drifts 1e-15 of its way, and the root of the discriminant A r^2 must
+  // not be that of a subnormal number, which is 0 here.
+  static constexpr float kAxial = 1e-30f;
   static constexpr float kPi = 3.14159265358979323846f;
   static constexpr float kTwoPi = 6.283185307179586f;
   static constexpr float kFourPi = 12.566370614359172f;
@@ -135,6 +139,7 @@ template <> struct Tr<double> {
   static __device__ __forceinline__ double quot(double a, double d) { return a / d; }
   static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
   static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+  static constexpr double kAxial = 0.0;
   static constexpr double kPi = 3.14159265358979323846;
   static constexpr double kTwoPi = 6.283185307179586;
   static constexpr double kFourPi = 12.566370614359172;
@@ -397,7 +402,7 @@ __device__ __forceinline__ Quad<R> quad(const R q[3], const R v[3], bool tube) {
 // is the better one; keeping them keeps every path as it was.
 template <bool FUSED, typename R>
 __device__ __forceinline__ bool hit_terms(const Quad<R>& Q, R r, R* qq, R* C) {
-  if (Q.A <= R(0)) return false;
+  if (Q.A <= Tr<R>::kAxial) return false;
   const R disc = Tr<R>::fma(Tr<R>::mul(Q.A, r), r, -Q.cross2);
   if (disc < R(0)) return false;
   *qq = -(Q.B + copysign(Tr<R>::root(disc), Q.B));
@@ -531,7 +536,7 @@ __device__ R entry_dist(const DPrim<R>& p, R dR, const R x[3], const R u[3], int
   const Quad<R> Q = quad(q, v, tube);
   const R div_A = Tr<R>::divisor(Q.A);
   R o0, o1;
-  if (Q.A == R(0)) {
+  if (Q.A <= Tr<R>::kAxial) {
     if (Q.C2 > rr.r1 * rr.r1) return INF;
     o0 = -INF; o1 = INF;
   } else if (!hit_radius<false>(Q, div_A, rr.r1, &o0, &o1)) {
@@ -552,9 +557,9 @@ __device__ R entry_dist(const DPrim<R>& p, R dR, const R x[3], const R u[3], int
   int f0 = 0, f1 = 1;
   if (rr.r0 > R(0)) {
     R i0, i1;
-    if (Q.A > R(0) && hit_radius<true>(Q, div_A, rr.r0, &i0, &i1)) {
+    if (hit_radius<true>(Q, div_A, rr.r0, &i0, &i1)) {
       e0 = i0; s1 = i1; e1 = o1;
-    } else if (Q.A == R(0) && Q.C2 < rr.r0 * rr.r0) {
+    } else if (Q.A <= Tr<R>::kAxial && Q.C2 < rr.r0 * rr.r0) {
       return INF;
     }
   }
