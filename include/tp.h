@@ -345,8 +345,9 @@ tp_status tp_backward(tp_scene* s, const double* grad_tallies, double* grad_para
                       void* stream);
 
 /* Replaces the instance parameters ([n_instances][n_params], same layout as
- * tp_scene_desc.inst_params) and re-validates the geometry (TP_ERR_GEOMETRY
- * leaves the old values in place).  Tallies are not reset. */
+ * tp_scene_desc.inst_params) and, where a primitive is bound to the radius,
+ * re-validates the geometry (TP_ERR_GEOMETRY leaves the old values in place).
+ * Tallies are not reset. */
 tp_status tp_set_params(tp_scene* s, const double* inst_params);
 
 /* Zeroes every tally and history count. */

@@ -121,3 +121,26 @@ def test_reset_runs_and_reads_on_several_streams_are_ordered():
     assert m0.any() and np.allclose(m1, m0, rtol=1e-11, atol=1e-11 * m0.max())
     # a gradient's terms cancel: rounding against the sum of their magnitudes, below 100 a history
     assert np.allclose(g1, g0, rtol=0.0, atol=1e-9)
+
+
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("prims", [10, 60])   # without and with a grid
+def test_parameters_that_move_nothing_change_on_a_scene_that_has_run(prims, graph):
+    """New densities (the geometry and its tables stay as they are), refused values
+    between, then densities back: each run is that of a scene made with them."""
+    from paper_2304_06226_gb300.engine import Scene
+    desc = W.imaging(n_prims=prims, precision="f64", psd_bins=16)
+    sc = Scene(desc)
+    for dens in (None, (0.5, 2.0, 1.5), (1.0, 1.0, 1.0)):
+        ref = copy.deepcopy(desc)
+        if dens is not None:
+            ref["instances"]["params"] = np.array([dens])
+            sc.set_params(np.array([dens]))
+            for bad in (np.nan, 0.0, -1.0):
+                with pytest.raises(RuntimeError):
+                    sc.set_params(np.array([[1.7, 1.7, bad]]))
+        sc.reset()
+        sc.run(N, kernel=1, graph=graph)
+        torch.cuda.synchronize()
+        same(sc, fresh(ref))
+    sc.close()
