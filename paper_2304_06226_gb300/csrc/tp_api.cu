@@ -893,7 +893,9 @@ tp_status pick_launch(tp_scene* s, bool grad, int req_block, int req_ctas, int* 
 
 // Bins of a histogram in shared memory: 16 KB a block leave FP32 warp pools
 // with tables of up to 3 KB their four blocks of 256 threads per SM (54 of 57 KB
-// a block); FP64 pools (55 KB without it) and larger tables keep three.
+// a block); FP64 pools (55 KB without it) and larger tables keep three, which still
+// pays (powder with 17 KB of tables, 1e7 histories: 1.69 ms counting with three
+// blocks, 1.96 ms summing with four).
 constexpr int kCountBinsMax = 4096;
 
 // A crossing scores at most twice in one bin.  A warp empties its block's histogram

@@ -59,9 +59,9 @@ constexpr unsigned kFull = 0xffffffffu;
 // tallies are histograms of counts in shared memory, see score.
 // kOptUnroll (80-register FP32 build of the plain history kernel): the group
 // sum's loop is left to the compiler's unrolling.  There it pays (guide of 2e7
-// histories 6.22 -> 5.75 ms, with powder the same and total scattering 2.02 -> 2.08 ms);
-// the 64-register build and the other kernels are better off with the short
-// loop (powder 3.28 against 3.43 ms, guide 5.38 against 5.52 ms).
+// histories 6.22 -> 5.74 ms, powder of 1e7 3.63 -> 3.61 ms, total scattering of 5e6
+// 2.02 -> 2.08 ms); the 64-register build is better off with the short loop
+// (powder 3.28 against 3.43 ms, guide 5.38 against 5.52 ms).
 constexpr int kOptGrid = 1, kOptFull = 2, kOptNoSec = 4, kOptCount = 8, kOptUnroll = 16;
 
 // ---------------------------------------------------------------------------
@@ -874,10 +874,11 @@ __device__ __forceinline__ void score_out(const KParams<R>& kp, const DTally<R>*
 // With kOptCount every weight is 1 (no process is biased and nothing reflects),
 // so sum w and sum w^2 of a bin are both its count: a score is one shared-memory
 // increment of 32 bits, and a block adds its counts to the two FP64 arrays when
-// it ends -- the same numbers, whole and exact.  Against two FP64 atomics in L2
-// for each group of lanes, and the match and the shuffles that find and sum the
-// groups: chopper study 1e7 histories 1.65 -> 0.67 ms, moderator 1e6 255 -> 144 us,
-// total scattering 1e7 2.14 -> 2.08 ms.
+// it ends -- the same numbers, whole and exact.  Summing takes two FP64 atomics
+// in L2 for each group of lanes, and the match and the shuffles that find and sum
+// the groups.  Warp pools with just over 4096 bins (summing) / just under
+// (counting): slit spectrum 1e6 histories 202 / 91 us, chopper 1e7 1.107 / 0.515 ms,
+// powder 1e8 16.7 / 13.3 ms, total scattering 1e7 1.89 / 1.69 ms.
 template <typename R, bool GRAD, int OPT>
 __device__ __forceinline__ void score(const KParams<R>& kp, const View<R>& V, const Particle<R>& P, unsigned mask,
                                       int face) {
@@ -1126,7 +1127,8 @@ __device__ __forceinline__ void entry_test(const View<R>& V, R dR, const R x[3],
 // round's loads are independent and a primitive's record is read only for its
 // entry test.  The walk's state is kept per axis in scalars: a run-time index
 // would put it into local memory.  Imaging of 1000 primitives, 2e7
-// histories: 16.5 -> 15.3 ms, with gradients 19.0 -> 18.4 ms.
+// histories: 16.5 -> 15.3 ms, with gradients 19.0 -> 18.4 ms a fit step (of which
+// 3 ms were host work that is gone since).
 template <typename R>
 __device__ __forceinline__ void grid_search(const KParams<R>& kp, const View<R>& V, R dR, R x0, R x1, R x2, R u0,
                                          R u1, R u2, int last, bool last_hull, R tmin, R* db_io, int* target_io,
@@ -1238,9 +1240,10 @@ struct Adv {
 // is (the regrouping kernels), which drops the other branch from the code.
 constexpr int kAny = 0, kInPrim = 1, kInWorld = 2;
 // For cross: either, with a mirror's reflection before the relocation instead of
-// inside it.  The warp pools run the scorer scenes 15 % and the guide 13 % faster
-// this way (5.29e9 against 4.62e9 histories/s total scattering, 1.05e10 against
-// 9.3e9 guide); the history kernel is 25 % slower on total scattering with it.
+// inside it.  The warp pools run the guide faster this way (1e8 histories 8.94
+// against 9.18 ms) and total scattering slower (4e7 6.43 against 6.22 ms); the
+// history kernel, for which it costs total scattering a tenth (4e7 16.5 against
+// 14.8 ms) and gains the guide nothing, does without.
 constexpr int kPoolCross = 3;
 
 template <typename R, bool GRAD, int OPT, int WHERE = kAny>
@@ -2126,25 +2129,26 @@ __global__ void __launch_bounds__(256, MINB) k_transport_ev(const __grid_constan
 // code path with most lanes busy.  Warps never wait for one another: no CTA
 // barrier after the table copy.
 //
-// What bounds it is the supply of instructions: a step runs some 650 of them
-// once each, the warps of an SM are at different places of the code, and the
-// fetch stall is the first of all (3.8 of 11 cycles an instruction on the powder
-// scene, 4.9 of 13 before).  Hence few of them: a step's slots come off a
-// stack, not out of a search of the pool, and a step writes back only the words
-// it changes.
+// What bounds it is the issue and the supply of instructions: a step runs some 600
+// of them once each, and the warps of an SM are at different places of the code.
+// In the lean build (powder) the schedulers issue in 80 % of the cycles and
+// waiting for a fetch is 1.6 of 10.0 cycles an instruction; in the full build
+// (total scattering) it is the first stall, 5.5 of 13.8, and so in gradient runs
+// with a radius parameter, 9.5 of 22.9.  Hence few instructions: a step's
+// slots come off a stack, not out of a search of the pool, and a step writes back
+// only the words it changes.
 //
 // Queues: each event type has a stack of slot numbers; the counts are one
 // packed word (a byte each) that every lane holds.  A step pops up to 32 slots
 // from the fullest stack and pushes each to the stack of its next event.  Last
 // in, first out keeps the neutrons of a step together -- started together,
 // they are mostly in the same volume and test the same surfaces.  Powder /
-// total scattering / guide / biased FP32 slab / imaging at 1e8, 4e7, 1e8, 4e7
-// and 1e7 histories, in 1e9 histories/s: 5.10 / 4.38 / 9.04 / 3.77 / 0.93 with
-// slots picked from the pool's event words by ballots and scoring at five
-// places, 5.78 / 5.29 / 10.5 / 4.12 / 1.05 with the stacks and one scoring
-// site; with the queues first in, first out 4.79 / 3.88 / 9.40 / 3.79 / 1.02;
-// with two warps of a sub-partition on a pool in common, so that one fetch may
-// serve both, 4.88 / 4.85 / 8.48 / 4.48 / 1.03.
+// total scattering / guide / biased FP32 slab at 1e8, 4e7, 1e8 and 4e7 histories
+// run at 7.55 / 6.22 / 11.2 / 4.12e9 histories/s.  Measured when the stacks were
+// made, before counting and the explicit geometry (stacks 5.78 / 5.29 / 10.5 /
+// 4.12): queues first in, first out 4.79 / 3.88 / 9.40 / 3.79; two warps of a
+// sub-partition on a pool in common, so that one fetch may serve both, 4.88 /
+// 4.85 / 8.48 / 4.48.
 // ---------------------------------------------------------------------------
 constexpr int kPool = 64;   // neutrons per warp (the stacks' counts are bytes)
 
