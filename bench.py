@@ -34,7 +34,7 @@ POWDER_N = 100_000_000
 # executes (ncu smsp__inst_executed.sum x active lanes / histories on a small
 # case of the same launch): an implementation's count, reported beside the
 # algorithmic one below.  Measured for the powder workload's warp-pool kernel.
-EXECUTED_INST_PER_HISTORY = {"powder": 3865}
+EXECUTED_INST_PER_HISTORY = {"powder": 3841}
 # Algorithmic lane operations of the method per step type, counted from its
 # formulas (not from any kernel):
 #   every event (biased flight, Eq. eStepLength2, and weight, Eq. eWeight):
@@ -62,11 +62,11 @@ def algorithmic_ops_per_history(counters: dict) -> float:
 # (ncu dram__bytes_read.sum + dram__bytes_write.sum), keyed by (workload,
 # variant): powder, the warp-pool launch (measured on 1e7 histories: the
 # tables' and tallies' cold misses, which do not grow with the histories);
-# batched, the two passes of a queued-secondaries step (measured on 4e6
-# histories of the same instance mix, the first pass on the event kernel, and
-# scaled by histories: the queue, written once and read once, makes it and grows
+# batched, the two passes of a queued-secondaries step, both on the warp pools
+# (measured on 4e6 histories of the same instance mix and scaled by histories: the
+# queue, written once and read once, and the first pass's spills make it and grow
 # with them).
-TRAFFIC_PER_LAUNCH = {("powder", 3): 120320, ("batched", 3): 246100000000}
+TRAFFIC_PER_LAUNCH = {("powder", 3): 121344, ("batched", 3): 284370000000}
 # The tally whose integrated total defines "matched tally error" per workload
 # (each history scores it at most once).
 FIGURE_TALLY = {"powder": 0, "guide": 0, "imaging": 0, "batched": 0, "slab": 1, "total_scattering": 1,
