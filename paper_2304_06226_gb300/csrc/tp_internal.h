@@ -80,7 +80,7 @@ template <typename R>
 struct alignas(4 * sizeof(R)) GridRow {
   R c[3], r;
 };
-// Rows the grid walk looks at in one round; the rows array has as many rows of
+// Rows the grid walk looks at in one round, at most; the rows array has as many rows of
 // padding after the last item.
 constexpr int kGridChunk = 4;
 

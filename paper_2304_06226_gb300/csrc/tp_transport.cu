@@ -1117,7 +1117,7 @@ __device__ __forceinline__ void entry_test(const View<R>& V, R dR, const R x[3],
 // World-region search through the uniform grid: a 3-D DDA over the cells the
 // ray crosses, nearest first, stopping once the best hit lies inside the cells
 // already visited.  One round of the walk takes, for a lane with no candidate
-// in hand, the next cell (or the next kGridChunk bounding spheres of a longer
+// in hand, the next cell (or the next kChunk bounding spheres of a longer
 // list) and, for a lane with candidates, the entry test of one of them.  Lanes
 // then meet at the long entry test in about as many rounds as the lane with
 // most cells and candidates needs (14 a step on the 1000-primitive scene);
@@ -1172,6 +1172,11 @@ __device__ __forceinline__ void grid_search(const KParams<R>& kp, const View<R>&
       tdel[a] = u[a] != R(0) ? fabs(Tr<R>::quot(kp.grid_cell[a], div_u[a])) : Tr<R>::inf();
     }
     int k = kp.grid_start[cell], k1 = kp.grid_start[cell + 1];
+    // (four FP64 rows are 32 registers: they spill, and a radiograph of 1000
+    // primitives, 2e5 histories, was slower than tested sphere by sphere, 5.56 ms
+    // against 5.50 on the history kernel and 4.75 against 4.71 on the pools; with
+    // two rows 5.27 and 4.53)
+    constexpr int kChunk = sizeof(R) == 8 ? 2 : kGridChunk;
     bool fresh = true;      // the cell's list is not looked at yet
     unsigned cand = 0;      // rows kb + i whose sphere is met, not yet tested
     int kb = 0;
@@ -1199,7 +1204,7 @@ __device__ __forceinline__ void grid_search(const KParams<R>& kp, const View<R>&
         kb = k;
         const R far = db * R(1.0001);
 #pragma unroll
-        for (int j = 0; j < kGridChunk; ++j) {
+        for (int j = 0; j < kChunk; ++j) {
           const GridRow<R> g = kp.grid_rows[k + j];
           // bounding sphere: pass over it if the ray misses it, moves away from
           // outside it, or meets it beyond the best hit (by more than rounding)
@@ -1210,7 +1215,7 @@ __device__ __forceinline__ void grid_search(const KParams<R>& kp, const View<R>&
           const bool miss = (qq > rb2 && (qu >= R(0) || Tr<R>::fma(-qu, qu, qq) > rb2)) || -qu - g.r > far;
           if (!miss && k + j < k1) cand |= 1u << j;
         }
-        k += kGridChunk;
+        k += kChunk;
       }
       if (cand != 0) {
         const int i = kp.grid_items[kb + __ffs(cand) - 1];
