@@ -1014,6 +1014,8 @@ cudaError_t launch_one(tp_scene* s, const LaunchCfg& c, bool grad, uint64_t seed
   k.regroup = c.regroup;
   const int grid = s->sm_count * c.ctas;
   const long long warps = (long long)grid * (c.block / 32);
+  const unsigned long long share = std::is_same<R, double>::value ? 4ull * s->sm_count : (unsigned long long)warps;
+  k.claim = sec_mode == 2 ? 32 : (int)std::max(1ull, std::min(32ull, total / share));
   k.hist_interval = (s->test_flags & TP_TEST_SMALL_HIST_INTERVAL) ? kHistIntervalTest : kHistInterval;
   k.chunk = sec_mode == 2 ? 16 : (int)std::max(1ll, std::min(256ll, (long long)(total / (unsigned long long)(warps * 8))));
   // the first launch after the run's description finds the counter at 0

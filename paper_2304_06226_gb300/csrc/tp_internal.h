@@ -126,6 +126,7 @@ struct KParams {
   unsigned long long total;
   unsigned long long* work_counter;
   int chunk;  // history kernel: histories a warp claims at once
+  int claim;              // warp pools: histories a warp starts with (FP64) or claims at most (FP32, grid)
   unsigned hist_interval;  // counting warp pools: crossings of a warp between emptyings of its block's histogram
   // event kernel, plain runs: the bank is regrouped every `regroup` events
   // (1 = every event); in between, each thread continues its own neutron

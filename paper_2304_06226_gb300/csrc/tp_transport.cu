@@ -2154,6 +2154,23 @@ __global__ void __launch_bounds__(256, MINB) k_transport_ev(const __grid_constan
 // 4.12): queues first in, first out 4.79 / 3.88 / 9.40 / 3.79; two warps of a
 // sub-partition on a pool in common, so that one fetch may serve both, 4.88 /
 // 4.85 / 8.48 / 4.48.
+//
+// Claims: a refill takes up to 32 histories from the work counter.  Two cases
+// have another rule (kp.claim, set by the host), because runs that do not fill
+// the chip would lie badly on it.
+//   FP64: a warp starts with kp.claim histories of its own, warp 0 of every
+// block before warp 1 of any; the counter serves what lies behind those.  A warp
+// instruction holds the FP64 pipe of its SM for some 18 cycles however many lanes
+// are active, so full warps, but on all SMs: the warps of the first blocks, which
+// ask first, would take all.  Histories a warp starts with: a quarter of an SM's
+// share, 32 at most.  Biased slab of 2e4 / 1e5 histories 668 / 774 -> 233 / 561 us,
+// powder of 3e3 205 -> 176 us, total scattering of 3e3 361 -> 180 us.
+//   FP32 on a grid: an even share of the run per warp, 32 at most.  A walk's
+// length differs from lane to lane, and few lanes wait for less: radiograph of
+// 600 primitives, 3e3 / 2e4 histories 141 / 201 -> 106 / 151 us.  Without a grid,
+// where a step is a fetch of its code first of all, full warps on few SMs are the
+// better ones (powder of 1e5 histories 92 us against 99 with 20 a claim and 100
+// with warps spread over the SMs).
 // ---------------------------------------------------------------------------
 constexpr int kPool = 64;   // neutrons per warp (the stacks' counts are bytes)
 
@@ -2267,7 +2284,7 @@ __global__ void __launch_bounds__(256, MINB) k_transport_wq(const __grid_constan
 #pragma unroll
   for (int i = 0; i < kPool; i += 32) stack[Q_EMPTY * kPool + i + lane] = (uint8_t)(i + lane);
   unsigned counts = (unsigned)kPool << (8 * Q_EMPTY);   // warp-uniform
-  bool work_left = true;                                // warp-uniform
+  bool work_left = true, started = false;               // warp-uniform
   unsigned emptied = 0;                                 // kOptCount: the warp's crossings at its last emptying
 
   for (;;) {
@@ -2286,7 +2303,13 @@ __global__ void __launch_bounds__(256, MINB) k_transport_wq(const __grid_constan
       }
     }
     // ---- lane j takes the j-th of the top entries ----
-    const int n = min(byte_of(counts, q), 32);
+    int n = min(byte_of(counts, q), 32);
+    const bool first = sizeof(R) == 8 && q == Q_EMPTY && !started;
+    if constexpr (sizeof(R) == 8) {
+      if (first) n = min(n, kp.claim);
+    } else if constexpr ((OPT & kOptGrid) != 0) {
+      if (q == Q_EMPTY) n = min(n, kp.claim);
+    }
     counts -= (unsigned)n << (8 * q);
     int slot = -1;
     if (lane < n) slot = stack[q * kPool + byte_of(counts, q) + lane];
@@ -2294,7 +2317,15 @@ __global__ void __launch_bounds__(256, MINB) k_transport_wq(const __grid_constan
     if (q == Q_EMPTY) {
       // new histories, claimed for the whole step at once
       unsigned long long g = 0;
-      if (lane == 0) g = aborted(kp, polls) ? total : atomicAdd(kp.work_counter, (unsigned long long)n);
+      if constexpr (sizeof(R) == 8) {
+        const unsigned long long nblk = gridDim.x, own = kp.claim;
+        g = first ? (warp * nblk + blockIdx.x) * own : (blockDim.x >> 5) * nblk * own;
+        started = true;
+      }
+      if (lane == 0) {
+        if (aborted(kp, polls)) g = total;
+        else if (!first) g += atomicAdd(kp.work_counter, (unsigned long long)n);
+      }
       g = __shfl_sync(kFull, g, 0) + lane;
       if (slot >= 0) {
         to = Q_EMPTY;

@@ -167,3 +167,25 @@ def test_histogram_emptied_while_the_block_scores(scene, precision, block):
     ref_cnt, ref = _run(desc, n, 2, 256)
     assert cnt == ref_cnt
     assert (got["sum"] == ref["sum"][0]).all() and (got["sumsq"] == ref["sumsq"][0]).all()
+
+
+@pytest.mark.parametrize("block,ctas", [(32, 1), (160, 0), (256, 0)])
+@pytest.mark.parametrize("n", [151, 609, 3001, 19_457, 20_011, 130_003])
+@pytest.mark.parametrize("scene,precision", [("slab", "f64"), ("chopper", "f64"), ("imaging", "f64"), ("imaging", "f32")])
+def test_every_history_is_claimed_once_whatever_the_share(scene, precision, n, block, ctas):
+    """Runs that end within the histories the warps start with, at their edge (19456 =
+    152 * 4 * 32 full warps) and beyond it; FP32 shares of a grid scene."""
+    from paper_2304_06226_gb300.engine import Scene
+    desc = {"slab": lambda: W.slab(g=3.0), "chopper": lambda: W.chopper(precision="f64"),
+            "imaging": lambda: W.imaging(n_prims=60, precision=precision, psd_bins=16)}[scene]()
+    seen = []
+    sc = Scene(desc)
+    for kernel in (1, 3):
+        sc.reset()
+        sc.run(n, kernel=kernel, block_size=block, ctas_per_sm=ctas)
+        torch.cuda.synchronize()
+        seen.append((sc.counters(), sc.raw()["sum"]))
+    sc.close()
+    assert seen[0][0] == seen[1][0] and seen[0][0]["histories"] == n
+    tol = 1e-12 if precision == "f64" else 1e-5   # (FP32: a group of up to 32 weights is summed in FP32)
+    assert np.allclose(seen[1][1], seen[0][1], rtol=tol, atol=tol * seen[0][1].max())
