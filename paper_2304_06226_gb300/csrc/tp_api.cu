@@ -143,7 +143,7 @@ struct tp_scene {
   uint32_t blob_bytes = 0;
   uint32_t off_prims = 0, off_mats = 0, off_mirrors = 0, off_choppers = 0, off_tallies = 0, off_line_d = 0,
            off_line_cum = 0, off_nb = 0;
-  bool blob_dirty = true;
+  bool blob_dirty = true, grid_dirty = true;   // the tables; the grid, which only primitives that move change
   // uniform grid (scenes with more than kGridMinPrims primitives)
   int* d_grid = nullptr;   // [ncells + 1] starts, then items
   void* d_grid_rows = nullptr;   // the items' bounding spheres (GridRow)
@@ -789,11 +789,14 @@ tp_status upload_blob(tp_scene* s) {
     cudaGraphExecDestroy(s->graph);
     s->graph = nullptr;
   }
-  tp_status gst = upload_grid(s);
+  tp_status gst = s->grid_dirty ? upload_grid(s) : TP_OK;
   if (gst != TP_OK) return gst;
   std::vector<uint8_t> blob = s->precision == TP_FP64 ? build_blob<double>(s) : build_blob<float>(s);
-  gst = s->precision == TP_FP64 ? upload_grid_rows<double>(s, blob) : upload_grid_rows<float>(s, blob);
-  if (gst != TP_OK) return gst;
+  if (s->grid_dirty) {
+    gst = s->precision == TP_FP64 ? upload_grid_rows<double>(s, blob) : upload_grid_rows<float>(s, blob);
+    if (gst != TP_OK) return gst;
+    s->grid_dirty = false;
+  }
   if (blob.size() > s->blob_cap) {
     if (s->d_blob) cudaFree(s->d_blob);
     s->d_blob = nullptr;
@@ -1483,7 +1486,7 @@ tp_status tp_set_params(tp_scene* s, const double* inst_params) {
   const std::vector<uint8_t> pb = params_bytes(s->inst_params, s->precision);
   TP_CUDA(cudaMemcpy(s->d_params, pb.data(), pb.size(), cudaMemcpyHostToDevice));
   s->default_work = true;
-  if (moving) s->blob_dirty = true;   // bounding radii and neighbour lists depend on the radii
+  if (moving) s->blob_dirty = s->grid_dirty = true;   // bounding radii and neighbour lists depend on the radii
   return TP_OK;
 }
 
