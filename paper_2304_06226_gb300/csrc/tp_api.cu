@@ -146,7 +146,7 @@ struct tp_scene {
   bool blob_dirty = true, grid_dirty = true;   // the tables; the grid, which only primitives that move change
   // uniform grid (scenes with more than kGridMinPrims primitives)
   int* d_grid = nullptr;   // [ncells + 1] starts, then items
-  void* d_grid_rows = nullptr;   // the items' bounding spheres (GridRow)
+  GridRow* d_grid_rows = nullptr;   // FP32: the items' bounding spheres
   std::vector<int> grid_items;   // host copy of the items
   int grid_n[3] = {0, 0, 0};
   double grid_lo[3] = {0, 0, 0}, grid_hi[3] = {0, 0, 0};
@@ -763,19 +763,18 @@ tp_status upload_grid(tp_scene* s) {
   return TP_OK;
 }
 
-// The bounding spheres of the grid's items, from the primitive records of the
+// FP32: the bounding spheres of the grid's items, from the primitive records of the
 // scene tables (the walk and the records then hold the same numbers).
-template <typename R>
 tp_status upload_grid_rows(tp_scene* s, const std::vector<uint8_t>& blob) {
-  if (s->grid_cells == 0) return TP_OK;
-  const auto* P = reinterpret_cast<const DPrim<R>*>(blob.data() + s->off_prims);
-  std::vector<GridRow<R>> rows(s->grid_items.size() + kGridChunk, GridRow<R>{});
+  if (s->grid_cells == 0 || s->precision != TP_FP32) return TP_OK;
+  const auto* P = reinterpret_cast<const DPrim<float>*>(blob.data() + s->off_prims);
+  std::vector<GridRow> rows(s->grid_items.size() + kGridChunk, GridRow{});
   for (size_t k = 0; k < s->grid_items.size(); ++k) {
-    const DPrim<R>& p = P[s->grid_items[k]];
-    rows[k] = GridRow<R>{{p.c[0], p.c[1], p.c[2]}, p.bound_r};
+    const DPrim<float>& p = P[s->grid_items[k]];
+    rows[k] = GridRow{{p.c[0], p.c[1], p.c[2]}, p.bound_r};
   }
-  TP_CUDA(cudaMalloc(&s->d_grid_rows, rows.size() * sizeof(GridRow<R>)));
-  TP_CUDA(cudaMemcpy(s->d_grid_rows, rows.data(), rows.size() * sizeof(GridRow<R>), cudaMemcpyHostToDevice));
+  TP_CUDA(cudaMalloc(&s->d_grid_rows, rows.size() * sizeof(GridRow)));
+  TP_CUDA(cudaMemcpy(s->d_grid_rows, rows.data(), rows.size() * sizeof(GridRow), cudaMemcpyHostToDevice));
   return TP_OK;
 }
 
@@ -793,7 +792,7 @@ tp_status upload_blob(tp_scene* s) {
   if (gst != TP_OK) return gst;
   std::vector<uint8_t> blob = s->precision == TP_FP64 ? build_blob<double>(s) : build_blob<float>(s);
   if (s->grid_dirty) {
-    gst = s->precision == TP_FP64 ? upload_grid_rows<double>(s, blob) : upload_grid_rows<float>(s, blob);
+    gst = upload_grid_rows(s, blob);
     if (gst != TP_OK) return gst;
     s->grid_dirty = false;
   }
@@ -870,7 +869,7 @@ void fill_common(const tp_scene* s, KParams<R>& k) {
   }
   k.grid_start = s->d_grid;
   k.grid_items = s->d_grid ? s->d_grid + s->grid_cells + 1 : nullptr;
-  k.grid_rows = static_cast<const GridRow<R>*>(s->d_grid_rows);
+  k.grid_rows = s->d_grid_rows;
   k.n_inst = s->n_inst;
   k.inst_prefix = s->d_prefix;
   k.inst_first = s->d_first;

@@ -73,14 +73,13 @@ struct alignas(16) DTally {
   int kind, trigger, volume, face, scat, nb0, nb1, offset;
 };
 
-// One entry of a grid cell's list: the bounding sphere of the primitive (its
-// centre and DPrim::bound_r), so that the walk reads the spheres of a cell from
+// One entry of a grid cell's list (FP32 walk): the bounding sphere of the primitive
+// (its centre and DPrim::bound_r), so that the walk reads the spheres of a cell from
 // consecutive rows.
-template <typename R>
-struct alignas(4 * sizeof(R)) GridRow {
-  R c[3], r;
+struct alignas(16) GridRow {
+  float c[3], r;
 };
-// Rows the grid walk looks at in one round, at most; the rows array has as many rows of
+// Rows the grid walk looks at in one round; the rows array has as many rows of
 // padding after the last item.
 constexpr int kGridChunk = 4;
 
@@ -114,7 +113,7 @@ struct KParams {
   R grid_lo[3], grid_hi[3], grid_cell[3], grid_inv[3];
   const int* grid_start;
   const int* grid_items;
-  const GridRow<R>* grid_rows;   // beside each item, its bounding sphere
+  const GridRow* grid_rows;   // FP32: beside each item, its bounding sphere
   // random numbers
   uint32_t key0, key1;
   int event_cap;

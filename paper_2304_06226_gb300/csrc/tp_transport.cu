@@ -1116,19 +1116,27 @@ __device__ __forceinline__ void entry_test(const View<R>& V, R dR, const R x[3],
 
 // World-region search through the uniform grid: a 3-D DDA over the cells the
 // ray crosses, nearest first, stopping once the best hit lies inside the cells
-// already visited.  One round of the walk takes, for a lane with no candidate
-// in hand, the next cell (or the next kChunk bounding spheres of a longer
-// list) and, for a lane with candidates, the entry test of one of them.  Lanes
-// then meet at the long entry test in about as many rounds as the lane with
-// most cells and candidates needs (14 a step on the 1000-primitive scene);
-// tested where each sphere was found, it ran for one or two lanes of the warp
-// at a time, some 34 times a step.  The spheres of a cell lie
-// beside one another (grid_rows, kGridChunk rows of padding at the end), so a
-// round's loads are independent and a primitive's record is read only for its
-// entry test.  The walk's state is kept per axis in scalars: a run-time index
-// would put it into local memory.  Imaging of 1000 primitives, 2e7
-// histories: 16.5 -> 15.3 ms, with gradients 19.0 -> 18.4 ms a fit step (of which
-// 3 ms were host work that is gone since).
+// already visited.
+//
+// FP32: one round of the walk takes, for a lane with no candidate in hand, the
+// next cell (or the next kGridChunk bounding spheres of a longer list) and, for a
+// lane with candidates, the entry test of one of them.  Lanes then meet at the
+// long entry test in about as many rounds as the lane with most cells and
+// candidates needs (14 a step on the 1000-primitive scene); tested where each
+// sphere was found, it ran for one or two lanes of the warp at a time, some 34
+// times a step.  The spheres of a cell lie beside one another (grid_rows,
+// kGridChunk rows of padding at the end), so a round's loads are independent and
+// a primitive's record is read only for its entry test.  The walk's state is kept
+// per axis in scalars: a run-time index would put it into local memory.  Imaging of
+// 1000 primitives, 2e7 histories: 16.5 -> 15.3 ms, with gradients 19.0 -> 18.4 ms a
+// fit step (of which 3 ms were host work that is gone since).
+//
+// FP64: each sphere's entry test where it is found.  The FP64 pipe is the bound;
+// rounds cull four spheres at a time in FP64, many of them past the cell's list, and
+// keep their rows in registers.  Radiographs, 5e5 histories, sphere by sphere
+// against rounds of two, history kernel / pools: 30 primitives 0.91 / 0.76 against
+// 1.12 / 0.94 ms, 100 2.06 / 1.63 against 2.27 / 1.80, 1000 10.2 / 7.4 against
+// 10.9 / 7.6.
 template <typename R>
 __device__ __forceinline__ void grid_search(const KParams<R>& kp, const View<R>& V, R dR, R x0, R x1, R x2, R u0,
                                          R u1, R u2, int last, bool last_hull, R tmin, R* db_io, int* target_io,
@@ -1171,59 +1179,67 @@ __device__ __forceinline__ void grid_search(const KParams<R>& kp, const View<R>&
       tnext[a] = u[a] != R(0) ? Tr<R>::quot(next, div_u[a]) : Tr<R>::inf();
       tdel[a] = u[a] != R(0) ? fabs(Tr<R>::quot(kp.grid_cell[a], div_u[a])) : Tr<R>::inf();
     }
-    int k = kp.grid_start[cell], k1 = kp.grid_start[cell + 1];
-    // (four FP64 rows are 32 registers: they spill, and a radiograph of 1000
-    // primitives, 2e5 histories, was slower than tested sphere by sphere, 5.56 ms
-    // against 5.50 on the history kernel and 4.75 against 4.71 on the pools; with
-    // two rows 5.27 and 4.53)
-    constexpr int kChunk = sizeof(R) == 8 ? 2 : kGridChunk;
-    bool fresh = true;      // the cell's list is not looked at yet
-    unsigned cand = 0;      // rows kb + i whose sphere is met, not yet tested
-    int kb = 0;
-    for (;;) {
-      if (cand == 0) {
-        if (!fresh && k >= k1) {
-          const R texit = fmin(tnext[0], fmin(tnext[1], tnext[2]));
-          if (db <= texit || texit >= t1) break;
-          // through the nearest face (the first of equals)
-          const bool a0 = tnext[0] <= tnext[1] && tnext[0] <= tnext[2];
-          const bool a1 = !a0 && tnext[1] <= tnext[2];
-          const int nl = (a0 ? left[0] : (a1 ? left[1] : left[2])) - 1;
-          if (nl < 0) break;
-          cell += a0 ? stp[0] : (a1 ? stp[1] : stp[2]);
-          left[0] = a0 ? nl : left[0];
-          left[1] = a1 ? nl : left[1];
-          left[2] = (a0 || a1) ? left[2] : nl;
-          tnext[0] = a0 ? tnext[0] + tdel[0] : tnext[0];
-          tnext[1] = a1 ? tnext[1] + tdel[1] : tnext[1];
-          tnext[2] = (a0 || a1) ? tnext[2] : tnext[2] + tdel[2];
-          k = kp.grid_start[cell];
-          k1 = kp.grid_start[cell + 1];
-        }
-        fresh = false;
-        kb = k;
-        const R far = db * R(1.0001);
+    // into the next cell, through the nearest face (the first of equals); false
+    // where the walk ends: at the best hit, the way's end or the grid's
+    auto next_cell = [&] {
+      const R texit = fmin(tnext[0], fmin(tnext[1], tnext[2]));
+      if (db <= texit || texit >= t1) return false;
+      const bool a0 = tnext[0] <= tnext[1] && tnext[0] <= tnext[2];
+      const bool a1 = !a0 && tnext[1] <= tnext[2];
+      const int nl = (a0 ? left[0] : (a1 ? left[1] : left[2])) - 1;
+      if (nl < 0) return false;
+      cell += a0 ? stp[0] : (a1 ? stp[1] : stp[2]);
+      left[0] = a0 ? nl : left[0];
+      left[1] = a1 ? nl : left[1];
+      left[2] = (a0 || a1) ? left[2] : nl;
+      tnext[0] = a0 ? tnext[0] + tdel[0] : tnext[0];
+      tnext[1] = a1 ? tnext[1] + tdel[1] : tnext[1];
+      tnext[2] = (a0 || a1) ? tnext[2] : tnext[2] + tdel[2];
+      return true;
+    };
+    if constexpr (sizeof(R) == 8) {
+      do {
+        const int k1 = kp.grid_start[cell + 1];
+        for (int k = kp.grid_start[cell]; k < k1; ++k)
+          entry_test(V, dR, x, u, kp.grid_items[k], last, last_hull, tmin, &db, &target, &face);
+      } while (next_cell());
+    } else {
+      int k = kp.grid_start[cell], k1 = kp.grid_start[cell + 1];
+      bool fresh = true;      // the cell's list is not looked at yet
+      unsigned cand = 0;      // rows kb + i whose sphere is met, not yet tested
+      int kb = 0;
+      for (;;) {
+        if (cand == 0) {
+          if (!fresh && k >= k1) {
+            if (!next_cell()) break;
+            k = kp.grid_start[cell];
+            k1 = kp.grid_start[cell + 1];
+          }
+          fresh = false;
+          kb = k;
+          const R far = db * R(1.0001);
 #pragma unroll
-        for (int j = 0; j < kChunk; ++j) {
-          const GridRow<R> g = kp.grid_rows[k + j];
-          // bounding sphere: pass over it if the ray misses it, moves away from
-          // outside it, or meets it beyond the best hit (by more than rounding)
-          const R q0 = x[0] - g.c[0], q1 = x[1] - g.c[1], q2 = x[2] - g.c[2];
-          const R qu = dot3(q0, u[0], q1, u[1], q2, u[2]);
-          const R qq = dot3(q0, q0, q1, q1, q2, q2);
-          const R rb2 = g.r * g.r;
-          const bool miss = (qq > rb2 && (qu >= R(0) || Tr<R>::fma(-qu, qu, qq) > rb2)) || -qu - g.r > far;
-          if (!miss && k + j < k1) cand |= 1u << j;
+          for (int j = 0; j < kGridChunk; ++j) {
+            const GridRow g = kp.grid_rows[k + j];
+            // bounding sphere: pass over it if the ray misses it, moves away from
+            // outside it, or meets it beyond the best hit (by more than rounding)
+            const R q0 = x[0] - g.c[0], q1 = x[1] - g.c[1], q2 = x[2] - g.c[2];
+            const R qu = dot3(q0, u[0], q1, u[1], q2, u[2]);
+            const R qq = dot3(q0, q0, q1, q1, q2, q2);
+            const R rb2 = g.r * g.r;
+            const bool miss = (qq > rb2 && (qu >= R(0) || Tr<R>::fma(-qu, qu, qq) > rb2)) || -qu - g.r > far;
+            if (!miss && k + j < k1) cand |= 1u << j;
+          }
+          k += kGridChunk;
         }
-        k += kChunk;
-      }
-      if (cand != 0) {
-        const int i = kp.grid_items[kb + __ffs(cand) - 1];
-        cand &= cand - 1;
-        if (!(i == last && last_hull)) {
-          int f;
-          const R t = entry_dist(V.prims[i], dR, x, u, &f, i == last ? tmin : R(0));
-          if (t < db) { db = t; target = i; face = f; }
+        if (cand != 0) {
+          const int i = kp.grid_items[kb + __ffs(cand) - 1];
+          cand &= cand - 1;
+          if (!(i == last && last_hull)) {
+            int f;
+            const R t = entry_dist(V.prims[i], dR, x, u, &f, i == last ? tmin : R(0));
+            if (t < db) { db = t; target = i; face = f; }
+          }
         }
       }
     }
