@@ -2323,15 +2323,17 @@ __global__ void __launch_bounds__(256, MINB) k_transport_wq(const __grid_constan
     const bool first = sizeof(R) == 8 && q == Q_EMPTY && !started;
     if constexpr (sizeof(R) == 8) {
       if (first) n = min(n, kp.claim);
-    } else if constexpr ((OPT & kOptGrid) != 0) {
-      if (q == Q_EMPTY) n = min(n, kp.claim);
     }
     counts -= (unsigned)n << (8 * q);
     int slot = -1;
     if (lane < n) slot = stack[q * kPool + byte_of(counts, q) + lane];
     int to = -1;   // queue of the slot's next event
     if (q == Q_EMPTY) {
-      // new histories, claimed for the whole step at once
+      // new histories, claimed for the whole step at once (shares: for the first
+      // m lanes, the other slots go back)
+      constexpr bool kShare = sizeof(R) == 4 && (OPT & kOptGrid);
+      int m = n;
+      if constexpr (kShare) m = min(n, kp.claim);
       unsigned long long g = 0;
       if constexpr (sizeof(R) == 8) {
         const unsigned long long nblk = gridDim.x, own = kp.claim;
@@ -2340,17 +2342,17 @@ __global__ void __launch_bounds__(256, MINB) k_transport_wq(const __grid_constan
       }
       if (lane == 0) {
         if (aborted(kp, polls)) g = total;
-        else if (!first) g += atomicAdd(kp.work_counter, (unsigned long long)n);
+        else if (!first) g += atomicAdd(kp.work_counter, (unsigned long long)m);
       }
       g = __shfl_sync(kFull, g, 0) + lane;
       if (slot >= 0) {
         to = Q_EMPTY;
-        if (g < total) {
+        if ((!kShare || lane < m) && g < total) {
           const int born = new_history<R, GRAD, OPT>(kp, V, pool, slot, g, cnt);
           if (born >= 0) to = born == 1 ? Q_ADVP : Q_ADVW;
         }
       }
-      work_left = __all_sync(kFull, slot < 0 || g < total) != 0;
+      work_left = __all_sync(kFull, (kShare ? lane >= m : slot < 0) || g < total) != 0;
       if constexpr ((OPT & kOptCount) != 0) {
         // long before a 32-bit count could run over (kHistInterval), the
         // histogram is emptied into the tallies
