@@ -63,9 +63,9 @@ def algorithmic_ops_per_history(counters: dict) -> float:
 # variant): powder, the warp-pool launch (measured on 1e7 histories: the
 # tables' and tallies' cold misses, which do not grow with the histories);
 # batched, the two passes of a queued-secondaries step, both on the warp pools
-# (measured on 4e6 histories of the same instance mix and scaled by histories: the
-# queue, written once and read once, and the first pass's spills make it and grow
-# with them).
+# (64-register build, measured on 4e6 histories of the same instance mix and
+# scaled by histories: the queue, written once and read once, and the first pass's
+# spills make it and grow with them).
 TRAFFIC_PER_LAUNCH = {("powder", 3): 121344, ("batched", 3): 284370000000}
 # The tally whose integrated total defines "matched tally error" per workload
 # (each history scores it at most once).
