@@ -1633,6 +1633,7 @@ tp_status tp_read_raw(tp_scene* s, int instance, double* sum, double* sumsq, dou
     if (J) TP_CUDA(cudaMemcpy(J + p * nb, s->d_J + src, nb * sizeof(double), kind));
     if (J2) TP_CUDA(cudaMemcpy(J2 + p * nb, s->d_J2 + src, nb * sizeof(double), kind));
   }
+  s->default_work = true;
   return TP_OK;
 }
 
