@@ -113,6 +113,7 @@ class Scene:
     def __init__(self, desc: dict, precision: str | None = None):
         self.desc = desc
         self._keep = []
+        self._side = False   # the last run lay on another stream than the default one
         prec = precision or desc.get("precision", "f32")
         d, keep = scene_struct(desc, prec)
         self._keep += keep
@@ -168,10 +169,12 @@ class Scene:
         fst = None if first is None else np.ascontiguousarray(
             np.broadcast_to(np.asarray(first, dtype=np.uint64), (self.n_inst,)))
         self._run_keep = (cnt, fst)
+        handle = _stream_handle(stream)
+        self._side = handle != 0
         r = N.tp_run(seed if seed is not None else self.seed,
                      cnt.ctypes.data_as(C.POINTER(C.c_uint64)),
                      None if fst is None else fst.ctypes.data_as(C.POINTER(C.c_uint64)),
-                     int(want_grad), _stream_handle(stream), block_size, ctas_per_sm,
+                     int(want_grad), handle, block_size, ctas_per_sm,
                      None if records is None else records.data_ptr(),
                      0 if records is None else records.numel() * records.element_size() // C.sizeof(N.tp_record),
                      kernel, int(graph), int(secondaries), int(regroup), int(stage))
@@ -182,6 +185,8 @@ class Scene:
         if device:
             mean = torch.empty(nb, dtype=torch.float64, device="cuda")
             err = torch.empty(nb, dtype=torch.float64, device="cuda")
+            if self._side:   # the read runs on the default stream: the buffers may come from another's past work
+                torch.cuda.current_stream().synchronize()
             N.tp_read_tallies(self.handle, t, instance, mean.data_ptr(), err.data_ptr(), True)
             torch.cuda.synchronize()
             return mean, err

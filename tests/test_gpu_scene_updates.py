@@ -144,3 +144,26 @@ def test_parameters_that_move_nothing_change_on_a_scene_that_has_run(prims, grap
         torch.cuda.synchronize()
         same(sc, fresh(ref))
     sc.close()
+
+
+def test_a_tally_read_on_a_side_stream_waits_for_the_work_its_buffers_come_from():
+    """The buffers of a read may be memory that earlier work of the side stream, freed
+    but not finished, still writes: it must not land in the result."""
+    from paper_2304_06226_gb300.engine import Scene
+    d = W.powder(precision="f64")
+    sc = Scene(d)
+    sc.run(N, kernel=1)
+    torch.cuda.synchronize()
+    want = sc.tally(0)[0].clone()
+    side, junk = torch.cuda.Stream(), torch.full((3600,), 7.0, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        sc.reset()
+        sc.run(N, kernel=1)
+        torch.cuda._sleep(20_000_000)                   # some ten milliseconds
+        parts = [junk.clone() for _ in range(8)]        # written after the wait, then given back
+        del parts
+        got = sc.tally(0)[0]
+        torch.cuda.synchronize()
+    assert torch.allclose(got, want, rtol=1e-11, atol=1e-11)
+    sc.close()
